@@ -7,104 +7,295 @@
 
 namespace lbm {
 
+// The fields of one cell that are averaged: the fixed-point phi, u and P = p / cs^2 - w0 (m.P) of
+// the propagated state, by the code of the time step: populations stay in storage units until
+// the moments, and only warps that hold a wall cell test their links against the walls.
 template <int Q, int S, bool GEN>
-__global__ void coarsen_kernel(const Params P, const void* __restrict__ fg, int f, float* __restrict__ out) {
+__device__ __forceinline__ void coarse_cell(const Params& P, const void* __restrict__ fg, int x, int y, int z, Macro& m,
+                                            int& phi_fx) {
+    const Nbr nb = make_nbr(P, x, y, z);
+    const int c = (z * P.ny + y) * P.nx + x;
+    const WallSide ws = GEN ? make_wall_side(P, x, y, z) : WallSide{};
+    float fb[Q], gb[Q];
+    const bool at_wall = GEN && (ws.xlo || ws.xhi || ws.ylo || ws.yhi || ws.zlo || ws.zhi);
+    if (GEN && __any_sync(__activemask(), at_wall))
+        pull<Q, true, S, true, true>(P, fg, c, nb, fb, gb, phi_fx, ws);
+    else
+        pull<Q, true, S, false, true>(P, fg, c, nb, fb, gb, phi_fx);
+    macro_flow<Q, GEN, S>(P, fb, gb, m);
+    macro_interface_df<Q, S>(P, m);
+    macro_pressure<GEN>(P, m);
+}
+
+// A sum of FP32 values held as an unevaluated pair (Knuth's two-sum: the rounding error of every
+// addition goes to lo), about 48 bits. GB300 issues an FP64 instruction per SM and 16 cycles for
+// a warp, so FP64 sums of four fields per cell (a conversion and an addition each) alone took as
+// long as the cell's bytes; a two-sum is seven FP32 instructions.
+struct Sum2 {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float v) {
+        const float s = __fadd_rn(hi, v), t = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(v, t)));
+        hi = s;
+    }
+    __device__ __forceinline__ void add(const Sum2& o) {
+        add(o.hi);
+        lo = __fadd_rn(lo, o.lo);
+    }
+    // the sum rounded once to FP32
+    __device__ __forceinline__ float rounded() const { return isfinite(hi) ? __fadd_rn(hi, lo) : hi; }
+    // where hi is infinite or NaN, lo is NaN and the sum is hi
+    __device__ __forceinline__ double value() const { return isfinite(hi) ? (double)hi + (double)lo : (double)hi; }
+};
+
+// The sums of a thread's cells: phi exactly in fixed point, u and P in pairs of FP32.
+struct CoarseSums {
+    long long phi = 0;
+    Sum2 v[4];  // u, P
+    __device__ __forceinline__ void add(const Macro& m, int phi_fx) {
+        phi += phi_fx;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) v[a].add(m.u[a]);
+        v[3].add(m.P);
+    }
+};
+
+// Means of n cells from their sums into coarse cell l of nc: p = cs^2 (w0 + mean P).
+__device__ __forceinline__ void store_means(const Params& P, long long phi, const double (&s)[4], double n,
+                                            float* __restrict__ out, long long nc, long long l) {
+    const double inv = 1.0 / n;
+    out[l] = (float)((double)phi * (inv / kPhiFx));
+#pragma unroll
+    for (int a = 0; a < 3; ++a) out[(1 + a) * nc + l] = (float)(s[a] * inv);
+    out[4 * nc + l] = (float)((P.w0d + s[3] * inv) / 3.0);
+}
+
+constexpr int kCoarseThreads = 128;
+
+// Register budgets as the time step's: the loads of a cell stay in flight at 4 blocks (FP32
+// storage, 128 registers) or 5 (16-bit, 96 registers) per SM. The periodic FP32 kernels that also
+// hold a thread's sums spill 84 bytes at 4 and take 3.
+template <int S, bool GEN, bool SUMS>
+constexpr int coarse_min_blocks() {
+    return S != STORE_F32 ? 5 : (SUMS && !GEN) ? 3 : 4;
+}
+
+// p = cs^2 (w0 + P) rounded to FP32 without an FP64 instruction, w0 = P.w0 + w0_lo: an exact sum,
+// and a division by 3 corrected by its remainder, rounds as the FP64 expression does but for ties.
+__device__ __forceinline__ float pressure_of(const Params& P, float w0_lo, const Sum2& mean) {
+    Sum2 w;
+    w.hi = P.w0;
+    w.lo = w0_lo;
+    w.add(mean);
+    constexpr float third = 1.0f / 3.0f;
+    const float q = w.hi * third;
+    const float r = fmaf(-3.0f, q, w.hi) + w.lo;
+    return isfinite(w.hi) ? fmaf(r, third, q) : w.hi;
+}
+
+// Factor 1: the fields of every cell. Bound by the state's bytes: 128^3 takes 61 us in FP32 (5.2 TB/s)
+// and 41 us in FP16 (4.1 TB/s), where FP64 sums and a division per cell took 203 and 187 us.
+template <int Q, int S, bool GEN>
+__global__ void __launch_bounds__(kCoarseThreads, (coarse_min_blocks<S, GEN, false>()))
+fields_kernel(const Params P, const void* __restrict__ fg, float w0_lo, float* __restrict__ out) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    const int z = blockIdx.z;
+    if (x >= P.nx || y >= P.ny) return;
+    Macro m;
+    int phi_fx;
+    coarse_cell<Q, S, GEN>(P, fg, x, y, z, m, phi_fx);
+    Sum2 dev;
+    dev.hi = m.P;
+    float* o = out + ((size_t)z * P.ny + y) * P.nx + x;
+    const size_t n = (size_t)P.N;
+    __stcs(o, __int2float_rn(phi_fx) * kPhiFxInvF);  // one rounding: 2^-30 is exact
+    __stcs(o + n, m.u[0]);
+    __stcs(o + 2 * n, m.u[1]);
+    __stcs(o + 3 * n, m.u[2]);
+    __stcs(o + 4 * n, pressure_of(P, w0_lo, dev));
+}
+
+// Block means over f^3 cells for factors f > 1 that divide 32: a block takes 32 consecutive fine x
+// of one coarse row, its four warps four of the f x f fine rows behind it at a time (neighbouring
+// rows together, so that they share their stencils in L1). phi is summed as integers and u in
+// pairs, so their order does not matter. The pressures are FP64 sums of rounded thirds, taken row
+// by row per lane and then across the f lanes of a coarse cell: their last bit depends on that
+// order, and a restart in 16-bit storage amplifies it, so it is fixed. The third of an FP64 value
+// is a product corrected by its remainder (the rounding of a division by 3, without its call),
+// which leaves six FP64 instructions per cell, fewer cycles than the rest of the cell.
+// f^3 is a power of two: the means of phi and u are FP32 roundings of their sums.
+// 256^3 at f = 4: 812 -> 380 us (FP16), 937 -> 613 us (FP32), at f = 2 925 -> 471 and 1018 -> 783 us; bound
+// by the propagation's instructions (16-bit) and its load latency (FP32).
+constexpr int kCoarseWarps = kCoarseThreads / 32;
+
+__device__ __forceinline__ double third_of(double x) {
+    constexpr double third = 1.0 / 3.0;
+    const double q = __dmul_rn(x, third);
+    const double t = fma(fma(-3.0, q, x), third, q);
+    return isfinite(t) ? t : q;
+}
+
+template <int Q, int S, bool GEN>
+__global__ void __launch_bounds__(kCoarseThreads, (coarse_min_blocks<S, GEN, true>()))
+coarsen_lanes_kernel(const Params P, const void* __restrict__ fg, int f, float* __restrict__ out) {
+    __shared__ float2 s_u[kCoarseWarps][3][32];
+    __shared__ long long s_phi[kCoarseWarps][32];
+    __shared__ double s_p[2][kCoarseWarps][32];
+    const int lane = threadIdx.x, warp = threadIdx.y;
+    const int x = blockIdx.x * 32 + lane, cy = blockIdx.y, cz = blockIdx.z;
+    const bool valid = x < P.nx;  // whole groups of f lanes are valid or not: f divides nx and 32
+    long long phi = 0;
+    Sum2 u[3];
+    double p = 0.0;  // in warp 0, of the lane's rows so far
+    for (int r0 = 0, k = 0; r0 < f * f; r0 += kCoarseWarps, k ^= 1) {  // f * f is a multiple of 4
+        if (valid) {
+            Macro m;
+            int phi_fx;
+            const int r = r0 + warp, dz = r / f;
+            coarse_cell<Q, S, GEN>(P, fg, x, cy * f + (r - dz * f), cz * f + dz, m, phi_fx);
+            phi += phi_fx;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) u[a].add(m.u[a]);
+            s_p[k][warp][lane] = third_of(P.w0d + (double)m.P);
+        }
+        __syncthreads();  // the other buffer is written only after every warp has passed the next one
+        if (warp == 0 && valid)
+            for (int w = 0; w < kCoarseWarps; ++w) p += s_p[k][w][lane];
+    }
+    s_phi[warp][lane] = phi;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) s_u[warp][a][lane] = make_float2(u[a].hi, u[a].lo);
+    __syncthreads();
+    if (warp != 0) return;
+    for (int w = 1; w < kCoarseWarps; ++w) {
+        phi += s_phi[w][lane];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            Sum2 o;
+            o.hi = s_u[w][a][lane].x;
+            o.lo = s_u[w][a][lane].y;
+            u[a].add(o);
+        }
+    }
+    for (int o = f >> 1; o > 0; o >>= 1) {
+        phi += __shfl_xor_sync(0xffffffffu, phi, o);
+        p += __shfl_xor_sync(0xffffffffu, p, o);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            Sum2 other;
+            other.hi = __shfl_xor_sync(0xffffffffu, u[a].hi, o);
+            other.lo = __shfl_xor_sync(0xffffffffu, u[a].lo, o);
+            u[a].add(other);
+        }
+    }
+    if (!valid || lane % f) return;
+    const float inv = 1.0f / (float)(f * f * f);
+    const int ncx = P.nx / f;
+    const long long nc = (long long)ncx * gridDim.y * gridDim.z;
+    float* o = out + ((long long)cz * gridDim.y + cy) * ncx + x / f;
+    o[0] = __ll2float_rn(phi) * (kPhiFxInvF * inv);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) o[(1 + a) * nc] = u[a].rounded() * inv;
+    o[4 * nc] = (float)(p * (double)inv);
+}
+
+// Any other factor up to kRowLanes: a block row of kRowLanes threads takes floor(kRowLanes / f)
+// whole coarse cells of one coarse row, each thread the f x f cells behind one fine x
+// (consecutive threads read consecutive cells), and one thread per coarse cell adds its f columns.
+// 192^3 FP32 at f = 3: 261 us, where one thread per coarse cell, which reads f cells apart, took 968 us; that
+// form stays for larger factors, whose blocks would hold no whole coarse cell.
+constexpr int kRowLanes = 64, kRowRows = kCoarseThreads / kRowLanes;
+
+template <int Q, int S, bool GEN>
+__global__ void __launch_bounds__(kCoarseThreads, (coarse_min_blocks<S, GEN, true>()))
+coarsen_rows_kernel(const Params P, const void* __restrict__ fg, int f, float* __restrict__ out) {
+    __shared__ double s_acc[kRowRows][4][kRowLanes];
+    __shared__ long long s_phi[kRowRows][kRowLanes];
+    const int t = threadIdx.x, r = threadIdx.y;
+    const int per = kRowLanes / f;  // coarse cells of a block row
+    const int x = blockIdx.x * per * f + t;
+    const int cy = blockIdx.y * kRowRows + r;
+    const int cz = blockIdx.z;
+    const int ncx = P.nx / f, ncy = P.ny / f, ncz = P.nz / f;
+    if (cy < ncy && t < per * f && x < P.nx) {
+        CoarseSums sums;
+        for (int dz = 0; dz < f; ++dz)
+            for (int dy = 0; dy < f; ++dy) {
+                Macro m;
+                int phi_fx;
+                coarse_cell<Q, S, GEN>(P, fg, x, cy * f + dy, cz * f + dz, m, phi_fx);
+                sums.add(m, phi_fx);
+            }
+        s_phi[r][t] = sums.phi;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) s_acc[r][k][t] = sums.v[k].value();
+    }
+    __syncthreads();
+    const int cx = blockIdx.x * per + t;
+    if (cy >= ncy || t >= per || cx >= ncx) return;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    long long phi = 0;
+    for (int j = t * f; j < (t + 1) * f; ++j) {
+        phi += s_phi[r][j];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc[k] += s_acc[r][k][j];
+    }
+    store_means(P, phi, acc, (double)f * f * f, out, (long long)ncx * ncy * ncz, ((long long)cz * ncy + cy) * ncx + cx);
+}
+
+template <int Q, int S, bool GEN>
+__global__ void __launch_bounds__(kCoarseThreads, (coarse_min_blocks<S, GEN, true>()))
+coarsen_cells_kernel(const Params P, const void* __restrict__ fg, int f, float* __restrict__ out) {
     const int cx = blockIdx.x * blockDim.x + threadIdx.x;
     const int cy = blockIdx.y * blockDim.y + threadIdx.y;
     const int cz = blockIdx.z;
     const int ncx = P.nx / f, ncy = P.ny / f, ncz = P.nz / f;
     if (cx >= ncx || cy >= ncy) return;
-    double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+    long long phi = 0;
     for (int dz = 0; dz < f; ++dz)
-        for (int dy = 0; dy < f; ++dy)
+        for (int dy = 0; dy < f; ++dy) {
+            CoarseSums sums;
             for (int dx = 0; dx < f; ++dx) {
-                const int x = cx * f + dx, y = cy * f + dy, z = cz * f + dz;
-                const Nbr nb = make_nbr(P, x, y, z);
-                const int c = (z * P.ny + y) * P.nx + x;
-                const WallSide ws = GEN ? make_wall_side(P, x, y, z) : WallSide{};
-                float fb[Q], gb[Q];
-                int phi_fx;
-                pull<Q, true, S, GEN>(P, fg, c, nb, fb, gb, phi_fx, ws);
                 Macro m;
-                macro_flow<Q, GEN>(P, fb, gb, m);
-                macro_interface_df<Q>(P, m);
-                macro_pressure<GEN>(P, m);
-                acc[0] += (double)phi_fx / kPhiFx;
-                acc[1] += m.u[0];
-                acc[2] += m.u[1];
-                acc[3] += m.u[2];
-                acc[4] += (P.w0d + (double)m.P) / 3.0;
+                int phi_fx;
+                coarse_cell<Q, S, GEN>(P, fg, cx * f + dx, cy * f + dy, cz * f + dz, m, phi_fx);
+                sums.add(m, phi_fx);
             }
-    const double inv = 1.0 / ((double)f * f * f);
-    const long long nc = (long long)ncx * ncy * ncz, l = ((long long)cz * ncy + cy) * ncx + cx;
-    for (int k = 0; k < 5; ++k) out[k * nc + l] = (float)(acc[k] * inv);
+            phi += sums.phi;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) acc[k] += sums.v[k].value();
+        }
+    store_means(P, phi, acc, (double)f * f * f, out, (long long)ncx * ncy * ncz, ((long long)cz * ncy + cy) * ncx + cx);
 }
 
-// The same block means for factors f that divide 32: lane l of a warp takes fine x = 32 b + l,
-// so a warp reads 32 consecutive cells of each plane, loops over the f x f rows of its coarse
-// cells and sums across each aligned group of f lanes (one coarse cell) with shuffles.
 template <int Q, int S, bool GEN>
-__global__ void coarsen_lanes_kernel(const Params P, const void* __restrict__ fg, int f, float* __restrict__ out) {
-    const int lane = threadIdx.x;
-    const int x = blockIdx.x * 32 + lane;
-    const int cy = blockIdx.y * blockDim.y + threadIdx.y;
-    const int cz = blockIdx.z;
+static void coarsen_qsg(const Params& P, const void* fg, int f, float* out, cudaStream_t s) {
     const int ncx = P.nx / f, ncy = P.ny / f, ncz = P.nz / f;
-    if (cy >= ncy) return;  // whole warps leave together
-    const bool valid = x < P.nx;  // whole groups of f lanes are valid or not: f divides nx and 32
-    double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    if (valid)
-        for (int dz = 0; dz < f; ++dz)
-            for (int dy = 0; dy < f; ++dy) {
-                const int y = cy * f + dy, z = cz * f + dz;
-                const Nbr nb = make_nbr(P, x, y, z);
-                const int c = (z * P.ny + y) * P.nx + x;
-                const WallSide ws = GEN ? make_wall_side(P, x, y, z) : WallSide{};
-                float fb[Q], gb[Q];
-                int phi_fx;
-                pull<Q, true, S, GEN>(P, fg, c, nb, fb, gb, phi_fx, ws);
-                Macro m;
-                macro_flow<Q, GEN>(P, fb, gb, m);
-                macro_interface_df<Q>(P, m);
-                macro_pressure<GEN>(P, m);
-                acc[0] += (double)phi_fx / kPhiFx;
-                acc[1] += m.u[0];
-                acc[2] += m.u[1];
-                acc[3] += m.u[2];
-                acc[4] += (P.w0d + (double)m.P) / 3.0;
-            }
-    for (int o = f >> 1; o > 0; o >>= 1)
-#pragma unroll
-        for (int k = 0; k < 5; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
-    if (!valid || lane % f) return;
-    const double inv = 1.0 / ((double)f * f * f);
-    const long long nc = (long long)ncx * ncy * ncz, l = ((long long)cz * ncy + cy) * ncx + x / f;
-    for (int k = 0; k < 5; ++k) out[k * nc + l] = (float)(acc[k] * inv);
+    const float w0_lo = (float)(P.w0d - (double)P.w0);
+    if (f == 1) {
+        const dim3 block = P.nx >= 128 ? dim3(128, 1) : dim3(32, 4);
+        const dim3 grid((P.nx + block.x - 1) / block.x, (P.ny + block.y - 1) / block.y, P.nz);
+        fields_kernel<Q, S, GEN><<<grid, block, 0, s>>>(P, fg, w0_lo, out);
+        return;
+    }
+    if constexpr (Q == 19) {  // D2Q9 grids have nz = 1, which only factor 1 divides
+        if (32 % f == 0) {
+            coarsen_lanes_kernel<Q, S, GEN><<<dim3((P.nx + 31) / 32, ncy, ncz), dim3(32, kCoarseWarps), 0, s>>>(P, fg, f, out);
+        } else if (f <= kRowLanes) {
+            const int per = kRowLanes / f;
+            coarsen_rows_kernel<Q, S, GEN><<<dim3((ncx + per - 1) / per, (ncy + kRowRows - 1) / kRowRows, ncz),
+                                             dim3(kRowLanes, kRowRows), 0, s>>>(P, fg, f, out);
+        } else {
+            coarsen_cells_kernel<Q, S, GEN><<<dim3((ncx + 31) / 32, (ncy + 3) / 4, ncz), dim3(32, 4), 0, s>>>(P, fg, f, out);
+    }
+    }
 }
 
 cudaError_t launch_coarsen(const Params& P, const void* fg, int factor, float* out, cudaStream_t s) {
-    const int ncx = P.nx / factor, ncy = P.ny / factor, ncz = P.nz / factor;
-    if (factor <= 32 && 32 % factor == 0) {
-        const dim3 block(32, 4), grid((P.nx + 31) / 32, (ncy + 3) / 4, ncz);
-#define LBM_COARSEN_LANES(Q, S)                                                                   \
-    (P.general ? (coarsen_lanes_kernel<Q, S, true><<<grid, block, 0, s>>>(P, fg, factor, out), 0) \
-               : (coarsen_lanes_kernel<Q, S, false><<<grid, block, 0, s>>>(P, fg, factor, out), 0))
-        if (P.Q == 9) {
-            if (P.storage == STORE_F16) LBM_COARSEN_LANES(9, STORE_F16);
-            else if (P.storage == STORE_BF16) LBM_COARSEN_LANES(9, STORE_BF16);
-            else LBM_COARSEN_LANES(9, STORE_F32);
-        } else {
-            if (P.storage == STORE_F16) LBM_COARSEN_LANES(19, STORE_F16);
-            else if (P.storage == STORE_BF16) LBM_COARSEN_LANES(19, STORE_BF16);
-            else LBM_COARSEN_LANES(19, STORE_F32);
-        }
-#undef LBM_COARSEN_LANES
-        return cudaGetLastError();
-    }
-    const dim3 block(32, 4), grid((ncx + 31) / 32, (ncy + 3) / 4, ncz);
-#define LBM_COARSEN(Q, S)                                                                   \
-    (P.general ? (coarsen_kernel<Q, S, true><<<grid, block, 0, s>>>(P, fg, factor, out), 0) \
-               : (coarsen_kernel<Q, S, false><<<grid, block, 0, s>>>(P, fg, factor, out), 0))
+#define LBM_COARSEN(Q, S) \
+    (P.general ? coarsen_qsg<Q, S, true>(P, fg, factor, out, s) : coarsen_qsg<Q, S, false>(P, fg, factor, out, s))
     if (P.Q == 9) {
         if (P.storage == STORE_F16) LBM_COARSEN(9, STORE_F16);
         else if (P.storage == STORE_BF16) LBM_COARSEN(9, STORE_BF16);
