@@ -11,8 +11,8 @@
  * Four periodic 3x3x3 convolutions, 5 -> 32 -> 32 -> 32 -> 5 channels, ReLU after the first
  * three; the prediction is input + output (a residual step). Convolutions accumulate in FP32;
  * activations between layers are stored in FP16 (or FP32, for gradient checks). With FP16
- * activations every layer (channels zero-padded to 32), its adjoint and its weight gradients
- * run on the tensor cores (tcgen05, FP16 operands, FP32 accumulation in tensor memory); in
+ * activations every layer (the five channels zero-padded to 8), its adjoint and its weight
+ * gradients run on the tensor cores (tcgen05, FP16 operands, FP32 accumulation in tensor memory); in
  * FP32 mode everything runs on the CUDA cores. A tensor-core wait that times out makes the
  * next synchronising call return LBM_ETIMEOUT. Weights are
  * FP32 ([Cout][Cin][27] then bias [Cout] per layer, tap = 9 dz + 3 dy + dx for the input offset

@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <cstring>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "../../include/lbm.h"
@@ -27,19 +28,22 @@ struct lbm_net {
     int cin[kLayers], cout[kLayers];
     long long w_off[kLayers], b_off[kLayers], n_params;
     float *params, *grads, *m, *v;   // device, n_params each
-    float* wt;                        // adjoint weights of one layer
-    __half* wimg;                     // FP16 tensor-core weight image of one 32 -> 32 layer
-    int* tc_err;                      // set by the tensor-core kernel if a wait timed out
-    long long tc_spin;                // polls of an mbarrier before a tensor-core wait for a step gives up
-    float* wscratch;                  // partial sums of the tensor-core weight gradients
+    float* wt;                        // FP32 mode: adjoint weights of one layer
+    // FP16 mode (tensor cores)
+    lbm::net::TcSizes tc;
+    void* images;                     // the layers' weights as operands
+    float *wgrad_part, *bias_part;    // partial sums of the gradients
+    int* tc_err;                      // set by a kernel if a wait timed out
+    long long tc_spin;                // polls of an mbarrier before a wait gives up
     int adam_step;
     float loss_w[kFieldChannels];     // per-channel weights of the loss
     // workspace for (batch, voxels)
     long long ws_elems;               // batch * voxels the workspace holds
-    void* x_t;                        // input in the activation type
     void* h[kLayers - 1];             // hidden activations
-    float* d;                         // last layer's output [B][5]
-    float *ga, *gb;                   // gradient ping-pong [B][32]
+    void *ga, *gb;                    // gradients of the hidden layers, ping-pong
+    float* d;                         // FP32 mode: last layer's output [B][5]
+    void *x_t, *gout;                 // FP16 mode: the input and the prediction's gradient, [B][vox][8]
+    unsigned int* bits[kLayers - 1];  // FP16 mode: which channels of h are positive
     double* partials;
     int n_partials;
     char err[512];
@@ -71,14 +75,19 @@ int nerr(lbm_net* n, int code, const char* fmt, ...) {
 
 void free_ws(lbm_net* n) {
     cudaFree(n->x_t);
-    for (int l = 0; l < kLayers - 1; ++l) cudaFree(n->h[l]);
+    cudaFree(n->gout);
+    for (int l = 0; l < kLayers - 1; ++l) {
+        cudaFree(n->h[l]);
+        cudaFree(n->bits[l]);
+        n->h[l] = nullptr;
+        n->bits[l] = nullptr;
+    }
     cudaFree(n->d);
     cudaFree(n->ga);
     cudaFree(n->gb);
     cudaFree(n->partials);
-    n->x_t = nullptr;
-    for (int l = 0; l < kLayers - 1; ++l) n->h[l] = nullptr;
-    n->d = n->ga = n->gb = nullptr;
+    n->x_t = n->gout = n->ga = n->gb = nullptr;
+    n->d = nullptr;
     n->partials = nullptr;
     n->ws_elems = 0;
 }
@@ -92,24 +101,31 @@ void free_net(lbm_net* n) {
     cudaFree(n->m);
     cudaFree(n->v);
     cudaFree(n->wt);
-    cudaFree(n->wimg);
+    cudaFree(n->images);
+    cudaFree(n->wgrad_part);
+    cudaFree(n->bias_part);
     cudaFree(n->tc_err);
-    cudaFree(n->wscratch);
     if (n->own_stream && n->stream) cudaStreamDestroy(n->stream);
     delete n;
 }
 
 int ensure_ws(lbm_net* n, int batch, long long vox) {
     const long long e = (long long)batch * vox;
-    const size_t act = n->fp16 ? 2 : 4;
     if (e <= n->ws_elems) return LBM_OK;
     free_ws(n);
-    LBM_NCUDA(n, cudaMalloc(&n->x_t, (size_t)e * kFieldChannels * act));
-    for (int l = 0; l < kLayers - 1; ++l) LBM_NCUDA(n, cudaMalloc(&n->h[l], (size_t)e * kHidden * act));
-    LBM_NCUDA(n, cudaMalloc(&n->d, (size_t)e * kFieldChannels * sizeof(float)));
-    LBM_NCUDA(n, cudaMalloc(&n->ga, (size_t)e * kHidden * sizeof(float)));
-    LBM_NCUDA(n, cudaMalloc(&n->gb, (size_t)e * kHidden * sizeof(float)));
-    n->n_partials = lbm::net::loss_blocks(e * kFieldChannels);
+    const size_t act = (size_t)e * kHidden * (n->fp16 ? 2 : 4);
+    for (int l = 0; l < kLayers - 1; ++l) LBM_NCUDA(n, cudaMalloc(&n->h[l], act));
+    LBM_NCUDA(n, cudaMalloc(&n->ga, act));
+    LBM_NCUDA(n, cudaMalloc(&n->gb, act));
+    if (n->fp16) {
+        LBM_NCUDA(n, cudaMalloc(&n->x_t, (size_t)e * 8 * 2));
+        LBM_NCUDA(n, cudaMalloc(&n->gout, (size_t)e * 8 * 2));
+        for (int l = 0; l < kLayers - 1; ++l) LBM_NCUDA(n, cudaMalloc(&n->bits[l], (size_t)e * sizeof(unsigned int)));
+        n->n_partials = n->tc.loss_parts;
+    } else {
+        LBM_NCUDA(n, cudaMalloc(&n->d, (size_t)e * kFieldChannels * sizeof(float)));
+        n->n_partials = lbm::net::loss_blocks(e * kFieldChannels);
+    }
     LBM_NCUDA(n, cudaMalloc(&n->partials, (size_t)n->n_partials * sizeof(double)));
     n->ws_elems = e;
     return LBM_OK;
@@ -138,10 +154,6 @@ int check_grid(lbm_net* n, int batch, const int grid[3]) {
     return LBM_OK;
 }
 
-// The layers run on the tensor cores with FP16 activations (channels zero-padded to 32); the FP32
-// mode stays on the CUDA-core kernels, whose results the gradient checks compare with FP64 at 1e-5.
-bool on_tensor_cores(const lbm_net* n) { return n->fp16 != 0; }
-
 // A timeout of the tensor-core kernel, read at a point where the stream has been synchronised.
 // The flag is cleared once reported, so the network stays usable: the kernel that timed out has
 // waited for its MMAs in flight and freed its tensor memory before it returned.
@@ -155,26 +167,47 @@ int check_tc(lbm_net* n) {
     return LBM_OK;
 }
 
-// Forward pass keeping the activations; the last layer's output in n->d.
+// FP16 mode: the network and its workspace as the tensor-core layers take them.
+lbm::net::TcNet tc_net(const lbm_net* n, int batch, const int grid[3]) {
+    lbm::net::TcNet t{};
+    t.params = n->params;
+    for (int l = 0; l < kLayers; ++l) {
+        t.cin[l] = n->cin[l];
+        t.cout[l] = n->cout[l];
+        t.w_off[l] = n->w_off[l];
+        t.b_off[l] = n->b_off[l];
+    }
+    t.batch = batch;
+    t.D = grid[2];
+    t.H = grid[1];
+    t.W = grid[0];
+    t.ctas = n->tc.ctas;
+    t.x = n->x_t;
+    for (int l = 0; l < kLayers - 1; ++l) {
+        t.h[l] = n->h[l];
+        t.bits[l] = n->bits[l];
+        t.g[l] = l & 1 ? n->gb : n->ga;
+    }
+    t.gout = n->gout;
+    t.images = n->images;
+    t.part = n->wgrad_part;
+    t.bias_part = n->bias_part;
+    t.loss_part = n->partials;
+    for (int c = 0; c < kFieldChannels; ++c) t.loss_w[c] = n->loss_w[c];
+    t.spin = n->tc_spin;
+    t.err = n->tc_err;
+    return t;
+}
+
+// FP32 mode: the forward pass keeping the activations; the last layer's output in n->d.
 int forward_keep(lbm_net* n, const float* x, int batch, const int grid[3]) {
     const int D = grid[2], H = grid[1], W = grid[0];
-    const long long vox = (long long)D * H * W;
-    int rc = ensure_ws(n, batch, vox);
-    if (rc) return rc;
-    LBM_NCUDA(n, lbm::net::cast_to(x, n->x_t, n->fp16, (long long)batch * kFieldChannels * vox, n->stream));
-    const void* in = n->x_t;
+    const float* in = x;
     for (int l = 0; l < kLayers; ++l) {
         const bool last = l == kLayers - 1;
-        void* out = last ? (void*)n->d : n->h[l];
-        if (on_tensor_cores(n)) {
-            LBM_NCUDA(n, lbm::net::weight_image(n->params + n->w_off[l], n->cout[l], n->cin[l], n->wimg, n->stream));
-            LBM_NCUDA(n, lbm::net::conv32_tc(in, 1, n->cin[l], 1.0f, n->wimg, n->params + n->b_off[l], out, last ? 0 : 1,
-                                             n->cout[l], last ? 0 : 1, batch, D, H, W, n->tc_spin, n->tc_err,
-                                             n->stream));
-        } else {
-            LBM_NCUDA(n, lbm::net::conv_forward(in, n->fp16, n->cin[l], n->params + n->w_off[l], n->params + n->b_off[l],
-                                                out, last ? 0 : n->fp16, n->cout[l], last ? 0 : 1, batch, D, H, W, n->stream));
-        }
+        float* out = last ? n->d : static_cast<float*>(n->h[l]);
+        LBM_NCUDA(n, lbm::net::conv_forward(in, n->cin[l], n->params + n->w_off[l], n->params + n->b_off[l], out, n->cout[l],
+                                            last ? 0 : 1, batch, D, H, W, n->stream));
         in = out;
     }
     return LBM_OK;
@@ -227,10 +260,15 @@ int lbm_net_create(lbm_net** out, int activations_fp16, unsigned long long seed,
     if (e == cudaSuccess) e = cudaMalloc(&n->grads, bytes);
     if (e == cudaSuccess) e = cudaMalloc(&n->m, bytes);
     if (e == cudaSuccess) e = cudaMalloc(&n->v, bytes);
-    if (e == cudaSuccess) e = cudaMalloc(&n->wt, (size_t)kHidden * kHidden * 27 * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&n->wimg, lbm::net::weight_image_bytes());
+    n->tc = lbm::net::tc_sizes();
+    if (n->fp16) {
+        if (e == cudaSuccess) e = cudaMalloc(&n->images, n->tc.image_bytes);
+        if (e == cudaSuccess) e = cudaMalloc(&n->wgrad_part, n->tc.part_floats * sizeof(float));
+        if (e == cudaSuccess) e = cudaMalloc(&n->bias_part, n->tc.bias_floats * sizeof(float));
+    } else if (e == cudaSuccess) {
+        e = cudaMalloc(&n->wt, (size_t)kHidden * kHidden * 27 * sizeof(float));
+    }
     if (e == cudaSuccess) e = cudaMalloc(&n->tc_err, sizeof(int));
-    if (e == cudaSuccess) e = cudaMalloc(&n->wscratch, lbm::net::wgrad_scratch_floats() * sizeof(float));
     if (e == cudaSuccess) e = cudaMemset(n->tc_err, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaMemcpy(n->params, h.data(), bytes, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(n->grads, 0, bytes);
@@ -268,10 +306,14 @@ int lbm_net_forward(lbm_net* n, const float* x, float* y, int batch, const int g
     if (!n || !x || !y) return nerr(n, LBM_EINVAL, "null argument");
     int rc = check_grid(n, batch, grid);
     if (rc) return rc;
-    rc = forward_keep(n, x, batch, grid);
-    if (rc) return rc;
-    const long long e = (long long)batch * kFieldChannels * grid[0] * grid[1] * grid[2];
-    LBM_NCUDA(n, lbm::net::residual(x, n->d, y, e, n->stream));
+    const long long vox = (long long)grid[0] * grid[1] * grid[2];
+    if ((rc = ensure_ws(n, batch, vox))) return rc;
+    if (n->fp16) {
+        LBM_NCUDA(n, lbm::net::tc_run(tc_net(n, batch, grid), x, y, nullptr, nullptr, nullptr, n->stream));
+        return LBM_OK;
+    }
+    if ((rc = forward_keep(n, x, batch, grid))) return rc;
+    LBM_NCUDA(n, lbm::net::residual(x, n->d, y, batch * kFieldChannels * vox, n->stream));
     return LBM_OK;
 }
 
@@ -279,42 +321,35 @@ int lbm_net_gradients(lbm_net* n, const float* x, const float* target, int batch
     if (!n || !x || !target) return nerr(n, LBM_EINVAL, "null argument");
     int rc = check_grid(n, batch, grid);
     if (rc) return rc;
-    rc = forward_keep(n, x, batch, grid);
-    if (rc) return rc;
     const int D = grid[2], H = grid[1], W = grid[0];
     const long long vox = (long long)D * H * W, e = (long long)batch * kFieldChannels * vox;
-    LBM_NCUDA(n, lbm::net::loss_and_grad(x, n->d, target, n->ga, e, vox, n->loss_w, n->partials, n->stream));
-    LBM_NCUDA(n, cudaMemsetAsync(n->grads, 0, (size_t)n->n_params * sizeof(float), n->stream));
-    float* g = n->ga;      // gradient of the current layer's output
-    float* other = n->gb;
-    const float grad_scale = std::ldexp(1.0f, std::ilogb((double)e));  // the power of two nearest below e
-    for (int l = kLayers - 1; l >= 0; --l) {
-        const void* h_in = (l == 0) ? n->x_t : n->h[l - 1];
-        if (on_tensor_cores(n))
-            LBM_NCUDA(n, lbm::net::wgrad32_tc(g, n->cout[l], grad_scale, h_in, n->fp16, n->cin[l], n->grads + n->w_off[l],
-                                              n->grads + n->b_off[l], batch, D, H, W, n->tc_spin, n->wscratch,
-                                              n->tc_err, n->stream));
-        else
-            LBM_NCUDA(n, lbm::net::conv_wgrad(g, n->cout[l], h_in, n->fp16, n->cin[l], n->grads + n->w_off[l],
-                                              n->grads + n->b_off[l], batch, D, H, W, n->stream));
-        if (l == 0) break;
-        LBM_NCUDA(n, lbm::net::flip_transpose(n->params + n->w_off[l], n->cout[l], n->cin[l], n->wt, n->stream));
-        if (on_tensor_cores(n)) {
-            LBM_NCUDA(n, lbm::net::weight_image(n->wt, n->cin[l], n->cout[l], n->wimg, n->stream));
-            // the loss gradient is 2 diff / (elements): scale it back to order one before FP16
-            LBM_NCUDA(n, lbm::net::conv32_tc(g, 0, n->cout[l], grad_scale, n->wimg, nullptr, other, 0, n->cin[l], 0, batch,
-                                             D, H, W, n->tc_spin, n->tc_err, n->stream));
-        } else {
-            LBM_NCUDA(n, lbm::net::conv_forward(g, 0, n->cout[l], n->wt, nullptr, other, 0, n->cin[l], 0, batch, D, H, W,
-                                                n->stream));
+    if ((rc = ensure_ws(n, batch, vox))) return rc;
+    int n_partials = n->n_partials;
+    if (n->fp16) {
+        lbm::net::TcNet t = tc_net(n, batch, grid);
+        // the loss gradient is 2 diff / (elements): scaled to order one before it is rounded to
+        // FP16, by the power of two nearest below the number of elements
+        t.grad_scale = std::ldexp(1.0f, std::ilogb((double)e));
+        LBM_NCUDA(n, lbm::net::tc_run(t, x, nullptr, target, n->grads, &n_partials, n->stream));
+    } else {
+        if ((rc = forward_keep(n, x, batch, grid))) return rc;
+        float *g = static_cast<float*>(n->ga), *other = static_cast<float*>(n->gb);  // of the current layer's output
+        n_partials = lbm::net::loss_blocks(e);
+        LBM_NCUDA(n, lbm::net::loss_and_grad(x, n->d, target, g, e, vox, n->loss_w, n->partials, n->stream));
+        LBM_NCUDA(n, cudaMemsetAsync(n->grads, 0, (size_t)n->n_params * sizeof(float), n->stream));
+        for (int l = kLayers - 1; l >= 0; --l) {
+            const float* h_in = (l == 0) ? x : static_cast<const float*>(n->h[l - 1]);
+            LBM_NCUDA(n, lbm::net::conv_wgrad(g, n->cout[l], h_in, n->cin[l], n->grads + n->w_off[l], n->grads + n->b_off[l],
+                                              batch, D, H, W, n->stream));
+            if (l == 0) break;
+            LBM_NCUDA(n, lbm::net::flip_transpose(n->params + n->w_off[l], n->cout[l], n->cin[l], n->wt, n->stream));
+            LBM_NCUDA(n, lbm::net::conv_forward(g, n->cout[l], n->wt, nullptr, other, n->cin[l], 0, batch, D, H, W, n->stream));
+            LBM_NCUDA(n, lbm::net::relu_mask(other, h_in, (long long)batch * n->cin[l] * vox, n->stream));
+            std::swap(g, other);
         }
-        LBM_NCUDA(n, lbm::net::relu_mask(other, n->h[l - 1], n->fp16, (long long)batch * n->cin[l] * vox, n->stream));
-        float* t = g;
-        g = other;
-        other = t;
     }
     if (loss) {
-        std::vector<double> part((size_t)n->n_partials);
+        std::vector<double> part((size_t)n_partials);
         LBM_NCUDA(n, cudaMemcpyAsync(part.data(), n->partials, part.size() * sizeof(double), cudaMemcpyDeviceToHost,
                                      n->stream));
         LBM_NCUDA(n, cudaStreamSynchronize(n->stream));

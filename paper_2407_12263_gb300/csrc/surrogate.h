@@ -3,7 +3,6 @@
 // Internal to the library.
 #pragma once
 
-#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include "lbm_internal.h"
@@ -15,18 +14,16 @@ constexpr int kFieldChannels = 5;  // phi, u, v, w, p
 constexpr int kHidden = 32;        // channels of the hidden layers
 constexpr int kLayers = 4;
 
-// Periodic 3x3x3 convolution of a batch [B][cin][D][H][W] into [B][cout][D][H][W]
-// (cout = 32 or 5), FP32 accumulation; inputs and outputs FP16 or FP32; relu on the output if
-// asked. bias may be NULL.
-cudaError_t conv_forward(const void* in, int in_fp16, int cin, const float* W, const float* bias, void* out, int out_fp16,
-                         int cout, int relu, int batch, int D, int H, int Wd, cudaStream_t s);
+// Periodic 3x3x3 convolution of a batch [B][cin][D][H][W] into [B][cout][D][H][W], FP32 on the
+// CUDA cores (cout = 32, or 5 without relu); relu on the output if asked. bias may be NULL.
+cudaError_t conv_forward(const float* in, int cin, const float* W, const float* bias, float* out, int cout, int relu, int batch,
+                         int D, int H, int Wd, cudaStream_t s);
 // gW [cout][cin][27] += correlation of g [B][cout] with h [B][cin]; gb [cout] += sum of g.
-cudaError_t conv_wgrad(const float* g, int cout, const void* h, int h_fp16, int cin, float* gW, float* gb, int batch,
-                       int D, int H, int Wd, cudaStream_t s);
+cudaError_t conv_wgrad(const float* g, int cout, const float* h, int cin, float* gW, float* gb, int batch, int D, int H, int Wd,
+                       cudaStream_t s);
 // Wt [cin][cout][27] with the taps reversed: the adjoint convolution's weights.
 cudaError_t flip_transpose(const float* W, int cout, int cin, float* Wt, cudaStream_t s);
-cudaError_t relu_mask(float* g, const void* h, int h_fp16, long long n, cudaStream_t s);
-cudaError_t cast_to(const float* x, void* y, int fp16, long long n, cudaStream_t s);
+cudaError_t relu_mask(float* g, const float* h, long long n, cudaStream_t s);
 cudaError_t residual(const float* x, const float* d, float* y, long long n, cudaStream_t s);
 int loss_blocks(long long n);
 // loss sum_i w_c(i) (x + d - target)_i^2 / n and its gradient; w: 5 host weights, vox: cells per channel.
@@ -34,29 +31,43 @@ cudaError_t loss_and_grad(const float* x, const float* d, const float* target, f
                           const float* w, double* partials, cudaStream_t s);
 cudaError_t adam(float* p, const float* g, float* m, float* v, long long n, float lr, int step, cudaStream_t s);
 
-// The 32 -> 32 convolution on the tensor cores (tcgen05): FP16 operands, FP32 accumulation.
-// wimg is the layer's weight image (weight_image, weight_image_bytes() bytes); inputs FP16 or
-// FP32, multiplied by in_scale (a power of two) before they are rounded to FP16 and the sums
-// divided by it again (so small gradients keep their bits); outputs FP16 with relu or FP32
-// without. *err is set to 1 if a wait for the tensor cores timed out: each wait for a step's
-// MMAs polls its mbarrier at most `spin` times, kTcWaitPolls normally or 0 (give up at once,
-// the same in every thread: a test of the timeout path); the last wait for MMAs still in
-// flight, before the tensor memory is freed, always allows kTcWaitPolls.
-// Layers with cin, cout <= 32 (the unused channels are zero-padded).
+// The layers on the tensor cores (tcgen05, surrogate_tc.cu): FP16 operands, FP32 accumulation. A
+// network's weights and the workspace of a batch, all device memory unless said otherwise.
+// Activations and gradients between layers are FP16, channels last; the five field channels are
+// padded to eight. *err is set to 1 if a wait gave up: each wait polls its mbarrier at most
+// `spin` times, kTcWaitPolls normally or 0 (give up at once, the same in every thread: a test of
+// the timeout path); the last wait for MMAs still in flight, before the tensor memory is freed,
+// always allows kTcWaitPolls.
 constexpr long long kTcWaitPolls = 1ll << 26;
-size_t weight_image_bytes();
-cudaError_t weight_image(const float* W, int cout, int cin, __half* img, cudaStream_t s);
-cudaError_t conv32_tc(const void* in, int in_fp16, int cin, float in_scale, const __half* wimg, const float* bias, void* out,
-                      int out_fp16, int cout, int relu, int batch, int D, int H, int Wd, long long spin, int* err,
-                      cudaStream_t s);
-// gW [cout][cin][27] += correlation of g [B][cout] with h [B][cin] on the tensor cores (g scaled by
-// g_scale, a power of two, before FP16 rounding and unscaled after); gb [cout] += sum of g.
-// scratch: wgrad_scratch_floats() floats of device memory for the per-CTA and per-block partial
-// sums, which are added in a fixed order: the gradients are the same bits on every run.
-constexpr int kBiasParts = 256;
-size_t wgrad_scratch_floats();
-cudaError_t wgrad32_tc(const float* g, int cout, float g_scale, const void* h, int h_fp16, int cin, float* gW, float* gb,
-                       int batch, int D, int H, int Wd, long long spin, float* scratch, int* err, cudaStream_t s);
+struct TcNet {
+    const float* params;
+    int cin[kLayers], cout[kLayers];
+    long long w_off[kLayers], b_off[kLayers];
+    int batch, D, H, W;
+    int ctas;                       // SMs of the device (tc_sizes)
+    void* x;                        // [B][vox][8]
+    void* h[kLayers - 1];           // [B][vox][32], outputs of the hidden layers
+    uint32_t* bits[kLayers - 1];    // [B][vox], bit c: channel c of h is positive (gradients only)
+    void* gout;                     // [B][vox][8], gradient of the prediction
+    void* g[kLayers - 1];           // [B][vox][32], gradients of the hidden layers; g[0] and g[2] may be one buffer
+    void* images;                   // tc_sizes().image_bytes: the weights as operands
+    float* part;                    // part_floats: the CTAs' weight-gradient sums
+    float* bias_part;               // bias_floats
+    double* loss_part;              // loss_parts doubles
+    float grad_scale;               // power of two that gradients are multiplied by before they are rounded to FP16
+    float loss_w[kFieldChannels];
+    long long spin;
+    int* err;
+};
+struct TcSizes {
+    int ctas, loss_parts;
+    size_t image_bytes, part_floats, bias_floats;
+};
+TcSizes tc_sizes();  // of the current device
+// target NULL: y = x + net(x). Otherwise the loss sum w_c (x + net(x) - target)^2 as *loss_parts
+// (host) partial sums in loss_part, and its mean's gradients with respect to all parameters in
+// grads. Partial sums are added in a fixed order: the same bits on every run.
+cudaError_t tc_run(const TcNet& N, const float* x, float* y, const float* target, float* grads, int* loss_parts, cudaStream_t s);
 
 }  // namespace net
 
