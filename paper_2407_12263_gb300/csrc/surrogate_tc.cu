@@ -92,6 +92,17 @@ __device__ __forceinline__ bool wait_parity(uint32_t mbar, uint32_t parity, long
     return false;
 }
 
+// Whether that phase has completed, without waiting for it.
+__device__ __forceinline__ bool test_parity(uint32_t mbar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred P1;\n\tmbarrier.test_wait.parity.shared::cta.b64 P1, [%1], %2;\n\tselp.b32 %0, 1, 0, P1;\n\t}\n"
+        : "=r"(ok)
+        : "r"(mbar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 // One thread of the (converged) warp. Only under elect.sync does the compiler know that the
 // issuing code is uniform and keeps descriptors in uniform registers: 39 cycles per MMA of N <= 32
 // against 48 for a branch on the thread index.
@@ -146,20 +157,20 @@ __device__ __forceinline__ void tmem_free(uint32_t tmem) {
 // ---------------------------------------------------------------------------------------
 struct Tiling {
     int D, H, W, tiles_x, tiles_y, most;
-    long long planes;
+    int planes;  // fewer than the grid's voxels, whose arrays fit the device
 };
 struct Column {
     int b, x0, y0, z0, nz;
 };
 struct Walk {
-    long long p, end;
+    int p, end;
     __device__ __forceinline__ explicit Walk(const Tiling& T)
-        : p(T.planes * blockIdx.x / gridDim.x), end(T.planes * (blockIdx.x + 1) / gridDim.x) {}
+        : p((int)((long long)T.planes * blockIdx.x / gridDim.x)), end((int)((long long)T.planes * (blockIdx.x + 1) / gridDim.x)) {}
     __device__ __forceinline__ bool next(const Tiling& T, Column& c) {
         if (p >= end) return false;
-        int tile = (int)(p / T.D);
-        c.z0 = (int)(p - (long long)tile * T.D);
-        const int n = (int)min(end - p, (long long)(T.D - c.z0));
+        int tile = p / T.D;
+        c.z0 = p - tile * T.D;
+        const int n = min(end - p, T.D - c.z0);
         const int parts = (n + T.most - 1) / T.most;
         c.nz = (n + parts - 1) / parts;
         c.x0 = (tile % T.tiles_x) * TX;
@@ -190,9 +201,12 @@ struct Walk {
 // a timeout a thread raises *err and the CTA's fail flag, all roles leave, the issuer waits once
 // more, with the full bound, for its MMAs, and the tensor memory is freed.
 //
-// Bound by shared memory: the MMAs' operands are 1015 cycles per plane of 128 voxels, the rest is
-// copies. Batch 4 at 64^3, 32 -> 32 channels: 53 us (1100 TFLOP/s of the layer's own multiply-adds;
-// 174 us with N = 32, planes staged through registers and block barriers between steps).
+// Bound by shared memory and L1: the MMAs' operands are 1015 cycles per plane of 128 voxels, the rest is
+// copies and stores. Batch 4 at 64^3, 32 -> 32 channels: 48 us (1200 TFLOP/s of the layer's own
+// multiply-adds; 174 us with N = 32, planes staged through registers and block barriers between
+// steps). Asking for the next plane while MMAs are queued, releasing accumulators one by one and
+// storing whole rows took it from 53 us; copies through registers, more copying warps and
+// announcing copies by their own completion made no difference or cost 3 to 15 us.
 // ---------------------------------------------------------------------------------------
 constexpr int kHx = TX + 2, kHy = TY + 2, kHaloed = kHx * kHy;
 // Bytes between chunk planes: 180 voxels x 16 and on to 32 modulo 128, so that the four 16-byte
@@ -266,6 +280,35 @@ struct LossSum {
     __device__ __forceinline__ double value() const { return far + ((double)hi + (double)lo); }
 };
 
+// The 64 bytes of every voxel of a warp (lane 8 y + x holds voxel (x0 + x, y0 + y)) to a plane of 32
+// channels. Lane bits 3 and 4 (y) change places with the 16-byte chunks, so that each store writes 8
+// whole voxels of one row, 512 consecutive bytes; a lane storing its own voxel 16 bytes at a time
+// took four times the passes through L1, which the copies and operands of the MMAs need.
+__device__ __forceinline__ void store_voxels(uint32_t (&v)[16], __half* plane, int x0, int y0, int H, int W) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int bit = 0; bit < 2; ++bit) {
+        const bool up = (lane >> (3 + bit)) & 1;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if ((k >> bit) & 1) continue;
+            const int lo = 4 * k, hi = 4 * (k | 1 << bit);  // chunks k and k + 2^bit
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                const uint32_t got = __shfl_xor_sync(0xffffffffu, up ? v[lo + w] : v[hi + w], 8 << bit);
+                if (up) v[lo + w] = got;
+                else v[hi + w] = got;
+            }
+        }
+    }
+    const int x = x0 + (lane & 7);
+    if (x >= W) return;
+    uint4* dst = reinterpret_cast<uint4*>(plane) + ((long long)y0 * W + x) * 4 + (lane >> 3);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        if (y0 + i < H) dst[(long long)i * W * 4] = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+}
+
 template <int KC, int NB, int MODE>
 __global__ void __launch_bounds__(kConvThreads, 2) conv_tc_kernel(const __grid_constant__ ConvArgs A) {
     using Sh = ConvShape<KC, NB>;
@@ -273,8 +316,8 @@ __global__ void __launch_bounds__(kConvThreads, 2) conv_tc_kernel(const __grid_c
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char* s_ring = smem;
     unsigned char* s_w = smem + kRing * Sh::kSlot;
-    // full[4], empty[4], done[8] (block finished), free (column drained), weights, drain
-    __shared__ __align__(8) unsigned long long s_bar[kRing * 2 + kMaxPlanes + 3];
+    // full[4], empty[4], done[8] (block finished), freed[8] (block read out), weights, drain
+    __shared__ __align__(8) unsigned long long s_bar[kRing * 2 + kMaxPlanes * 2 + 2];
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_fail;
     const int t = threadIdx.x, warp = __shfl_sync(0xffffffffu, t / 32, 0);
@@ -282,14 +325,17 @@ __global__ void __launch_bounds__(kConvThreads, 2) conv_tc_kernel(const __grid_c
     auto full = [&](int s) { return bar + 8u * (uint32_t)s; };
     auto empty = [&](int s) { return bar + 8u * (uint32_t)(kRing + s); };
     auto done = [&](int o) { return bar + 8u * (uint32_t)(2 * kRing + o); };
-    const uint32_t bar_free = bar + 8u * (2 * kRing + kMaxPlanes), bar_w = bar_free + 8, bar_drain = bar_free + 16;
+    auto freed = [&](int o) { return bar + 8u * (uint32_t)(2 * kRing + kMaxPlanes + o); };
+    const uint32_t bar_w = bar + 8u * (2 * kRing + 2 * kMaxPlanes), bar_drain = bar_w + 8;
     if (t == 0) {
         for (int s = 0; s < kRing; ++s) {
             mbar_init(full(s), kStagers);
             mbar_init(empty(s), 1);
         }
-        for (int o = 0; o < kMaxPlanes; ++o) mbar_init(done(o), 1);
-        mbar_init(bar_free, kEpiThreads);
+        for (int o = 0; o < kMaxPlanes; ++o) {
+            mbar_init(done(o), 1);
+            mbar_init(freed(o), kEpiThreads);
+        }
         mbar_init(bar_w, 1);
         mbar_init(bar_drain, 1);
         s_fail = 0;
@@ -323,18 +369,14 @@ __global__ void __launch_bounds__(kConvThreads, 2) conv_tc_kernel(const __grid_c
             const uint32_t ring = smem_u32(s_ring);
             const uint64_t b0 = smem_desc(smem_u32(s_w), Sh::kRows * 16, 128);
             bool ok = wait_parity(bar_w, 0, A.spin, &s_fail);
-            uint32_t q = 0, n_col = 0;  // planes and columns so far
+            uint32_t q = 0, used = 0, phase = 0;  // planes so far; per block: written before, parity of its next release
+            bool ready = false;                   // plane q is known to be there
             Walk walk(A.t);
-            for (Column c; ok && walk.next(A.t, c); ++n_col) {
+            for (Column c; ok && walk.next(A.t, c);) {
                 const int nz = c.nz;
-                if (n_col > 0) {  // the blocks of the column before are read out
-                    ok = wait_parity(bar_free, (n_col - 1) & 1, A.spin, &s_fail);
-                    if (!ok) break;
-                    fence_after();
-                }
                 for (int j = -1; j <= nz; ++j, ++q) {
                     const uint32_t s = q % kRing;
-                    ok = wait_parity(full(s), (q / kRing) & 1, A.spin, &s_fail);
+                    ok = ready || wait_parity(full(s), (q / kRing) & 1, A.spin, &s_fail);
                     if (!ok) break;
                     fence_after();
                     // plane j goes to the output planes j - 1 .. j + 1 that the column has
@@ -344,6 +386,13 @@ __global__ void __launch_bounds__(kConvThreads, 2) conv_tc_kernel(const __grid_c
                     const uint32_t d = tmem + (uint32_t)(lo * NB), n = (uint32_t)((hi - lo + 1) * NB);
                     const bool fresh = hi == j + 1;
                     if (fresh) {  // block hi starts here: its first product replaces what it held
+                        if ((used >> hi) & 1) {  // an output of the column before, which must have been read
+                            ok = wait_parity(freed(hi), (phase >> hi) & 1, A.spin, &s_fail);
+                            if (!ok) break;
+                            phase ^= 1u << hi;
+                            fence_after();
+                        }
+                        used |= 1u << hi;
                         if (lo < hi) mma_f16(d, a, b, kIdesc | idesc_n(n - NB), 1);
                         mma_f16(tmem + (uint32_t)(hi * NB), a, b + (uint64_t)((hi - lo) * NB), kIdesc | idesc_n(NB), 0);
                     } else {
@@ -351,12 +400,15 @@ __global__ void __launch_bounds__(kConvThreads, 2) conv_tc_kernel(const __grid_c
                     }
                     const uint32_t id = kIdesc | idesc_n(n);
 #pragma unroll
-                    for (int tap = 0; tap < 9; ++tap)
+                    for (int tap = 0; tap < 9; ++tap) {
+                        // asked while MMAs are queued: the answer's latency leaves no gap between planes
+                        if (tap == 6) ready = test_parity(full((q + 1) % kRing), ((q + 1) / kRing) & 1);
 #pragma unroll
                         for (int k = 0; k < Sh::kSteps; ++k)
                             if (tap || k)
                                 mma_f16(d, a + (uint64_t)((tap / 3) * kHx + tap % 3 + k * (int)(2 * kChunk / 16)),
                                         b + (uint64_t)((tap * (int)Sh::kTap + k * (int)(2 * Sh::kRows * 16)) / 16), id, 1);
+                    }
                     commit(empty(s));
                     if (j >= 1) commit(done(j - 1));
                 }
@@ -420,19 +472,31 @@ __global__ void __launch_bounds__(kConvThreads, 2) conv_tc_kernel(const __grid_c
         for (Column c; ok && walk.next(A.t, c);) {
             const int x = c.x0 + t % TX, y = c.y0 + t / TX;
             const bool inside = x < A.t.W && y < A.t.H;
+            // what an output needs besides its sums
+            struct Extra {
+                uint32_t bits;
+                float x[MODE == kPrediction || MODE == kLossGrad ? kFieldChannels : 1], t[MODE == kLossGrad ? kFieldChannels : 1];
+            } next;
+            auto fetch = [&](long long row, long long e) {
+                Extra f{};
+                if (!inside) return f;
+                if (MODE == kAdjoint) f.bits = __ldg(A.bits + row);
+                if (MODE == kPrediction || MODE == kLossGrad)
+#pragma unroll
+                    for (int ch = 0; ch < kFieldChannels; ++ch) {
+                        f.x[ch] = __ldg(A.x + e + ch * vox);
+                        if (MODE == kLossGrad) f.t[ch] = __ldg(A.target + e + ch * vox);
+                    }
+                return f;
+            };
             for (int o = 0; o < c.nz; ++o) {
                 const long long v = ((long long)(c.z0 + o) * A.t.H + y) * A.t.W + x;  // in its sample
                 const long long row = (long long)c.b * vox + v, e = (long long)c.b * kFieldChannels * vox + v;
-                // what the output needs besides its sums is read before they are waited for
-                uint32_t bits = 0;
-                float xs[kFieldChannels], ts[kFieldChannels];
-                if (MODE == kAdjoint && inside) bits = __ldg(A.bits + row);
-                if ((MODE == kPrediction || MODE == kLossGrad) && inside)
-#pragma unroll
-                    for (int ch = 0; ch < kFieldChannels; ++ch) {
-                        xs[ch] = __ldg(A.x + e + ch * vox);
-                        if (MODE == kLossGrad) ts[ch] = __ldg(A.target + e + ch * vox);
-                    }
+                if (o == 0) next = fetch(row, e);
+                const Extra now = next;
+                uint32_t bits = now.bits;
+                // read while this output is waited for and finished
+                if (o + 1 < c.nz) next = fetch(row + (long long)A.t.H * A.t.W, e + (long long)A.t.H * A.t.W);
                 if (!wait_parity(done(o), (phase >> o) & 1, A.spin, &s_fail)) {
                     ok = false;
                     break;
@@ -443,54 +507,46 @@ __global__ void __launch_bounds__(kConvThreads, 2) conv_tc_kernel(const __grid_c
                 if constexpr (NB == 32) {
                     uint32_t r[32];
                     tmem_load32(addr, r);
-                    if (o == c.nz - 1) {
-                        fence_before();
-                        mbar_arrive(bar_free);
-                    }
-                    if (inside) {
-                        uint32_t packed[16];
-                        if (MODE == kHiddenLayer) {
+                    fence_before();
+                    mbar_arrive(freed(o));
+                    uint32_t packed[16];
+                    if (MODE == kHiddenLayer) {
 #pragma unroll
-                            for (int i = 0; i < 16; ++i) {
-                                const __half2 p = __floats2half2_rn(fmaxf(__uint_as_float(r[2 * i]) + bias[2 * i], 0.f),
-                                                                    fmaxf(__uint_as_float(r[2 * i + 1]) + bias[2 * i + 1], 0.f));
-                                const uint32_t u = *reinterpret_cast<const uint32_t*>(&p);
-                                packed[i] = u;  // values are >= 0: positive is not zero
-                                bits |= ((u & 0x7fffu) ? 1u : 0u) << (2 * i) | ((u & 0x7fff0000u) ? 1u : 0u) << (2 * i + 1);
-                            }
-                            if (A.bits) A.bits[row] = bits;
-                        } else {
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) {
-                                const float a = (bits >> (2 * i)) & 1 ? __uint_as_float(r[2 * i]) : 0.f;
-                                const float b = (bits >> (2 * i + 1)) & 1 ? __uint_as_float(r[2 * i + 1]) : 0.f;
-                                sums[2 * i] += a;
-                                sums[2 * i + 1] += b;
-                                const __half2 p = __floats2half2_rn(a, b);
-                                packed[i] = *reinterpret_cast<const uint32_t*>(&p);
-                            }
+                        for (int i = 0; i < 16; ++i) {
+                            const __half2 p = __floats2half2_rn(fmaxf(__uint_as_float(r[2 * i]) + bias[2 * i], 0.f),
+                                                                fmaxf(__uint_as_float(r[2 * i + 1]) + bias[2 * i + 1], 0.f));
+                            const uint32_t u = *reinterpret_cast<const uint32_t*>(&p);
+                            packed[i] = u;  // values are >= 0: positive is not zero
+                            bits |= ((u & 0x7fffu) ? 1u : 0u) << (2 * i) | ((u & 0x7fff0000u) ? 1u : 0u) << (2 * i + 1);
                         }
-                        uint4* dst = reinterpret_cast<uint4*>(A.out + row * 32);
+                        if (A.bits && inside) A.bits[row] = bits;
+                    } else {
 #pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            dst[i] = make_uint4(packed[4 * i], packed[4 * i + 1], packed[4 * i + 2], packed[4 * i + 3]);
+                        for (int i = 0; i < 16; ++i) {  // outside the grid every bit is 0
+                            const float a = (bits >> (2 * i)) & 1 ? __uint_as_float(r[2 * i]) : 0.f;
+                            const float b = (bits >> (2 * i + 1)) & 1 ? __uint_as_float(r[2 * i + 1]) : 0.f;
+                            sums[2 * i] += a;
+                            sums[2 * i + 1] += b;
+                            const __half2 p = __floats2half2_rn(a, b);
+                            packed[i] = *reinterpret_cast<const uint32_t*>(&p);
+                        }
                     }
+                    store_voxels(packed, A.out + ((long long)c.b * vox + (long long)(c.z0 + o) * A.t.H * A.t.W) * 32, c.x0,
+                                 c.y0 + 4 * warp, A.t.H, A.t.W);
                 } else {
                     uint32_t r[8];
                     tmem_load8(addr, r);
-                    if (o == c.nz - 1) {
-                        fence_before();
-                        mbar_arrive(bar_free);
-                    }
+                    fence_before();
+                    mbar_arrive(freed(o));
                     if (inside) {
                         float g[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                         for (int ch = 0; ch < kFieldChannels; ++ch) {
                             const float d = __uint_as_float(r[ch]) + bias[ch];
                             if (MODE == kPrediction) {
-                                A.y[e + ch * vox] = xs[ch] + d;
+                                A.y[e + ch * vox] = now.x[ch] + d;
                             } else {
-                                const float diff = xs[ch] + d - ts[ch];
+                                const float diff = now.x[ch] + d - now.t[ch];
                                 g[ch] = A.loss_scale * A.w[ch] * diff;
                                 sums[ch] += g[ch];
                                 loss.add(A.w[ch], diff);
@@ -556,7 +612,7 @@ __global__ void __launch_bounds__(kConvThreads, 2) conv_tc_kernel(const __grid_c
 // ring of five; after unit j the MMAs of g's plane j - 1 with h's planes j - 2, j - 1, j run. Its sums
 // go to a slice of its own, added in CTA order by grads_finish_kernel.
 //
-// Bound as the convolution: batch 4 at 64^3, 32 x 32 channels, 60 us against 174 us (45 us against 174
+// Bound as the convolution: batch 4 at 64^3, 32 x 32 channels, 58 us against 174 us (45 us against 174
 // with the five fields on either side).
 // ---------------------------------------------------------------------------------------
 constexpr int kWgThreads = 256, kWgStagers = 224, kWgRing = 5;
@@ -628,12 +684,14 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
         if (elect_one()) {
             bool ok = true;
             uint32_t q = 0, acc = 0;
+            bool ready = false;  // unit q is known to be there
             constexpr uint32_t id = kIdesc | kMnMajor | idesc_n(Sh::kN);
             auto slot = [&](uint32_t back) { return (q + kWgRing - back) % kWgRing; };
             Walk walk(A.t);
             for (Column c; ok && walk.next(A.t, c);) {
                 for (int j = Sh::kFirst; j < c.nz + Sh::kPast; ++j, ++q) {
-                    ok = wait_parity(full(slot(0)), (q / kWgRing) & 1, A.spin, &s_fail);
+                    ok = ready || wait_parity(full(slot(0)), (q / kWgRing) & 1, A.spin, &s_fail);
+                    ready = false;
                     if (!ok) break;
                     fence_after();
                     if (!Sh::kStack && j < 1) continue;
@@ -642,9 +700,11 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
                     for (int dz = 0; dz < Sh::kAccs; ++dz) {
                         const uint64_t a = smem_desc(ring + slot(Sh::kAccs - 1 - dz) * Sh::kUnit, Sh::kRowA, Sh::kMatA);
 #pragma unroll
-                        for (int k = 0; k < TY / 2; ++k)  // two rows of 8 voxels per MMA
+                        for (int k = 0; k < TY / 2; ++k) {  // two rows of 8 voxels per MMA
+                            if (dz == Sh::kAccs - 1 && k == 4) ready = test_parity(full((q + 1) % kWgRing), ((q + 1) / kWgRing) & 1);
                             mma_f16(tmem + (uint32_t)(dz * Sh::kN), a + (uint64_t)(2 * k * (int)Sh::kRowA / 16),
                                     b + (uint64_t)(2 * k * (int)Sh::kRowB / 16), id, k ? 1u : acc);
+                        }
                     }
                     acc = 1;
                     if (Sh::kStack) {
@@ -856,7 +916,7 @@ int sm_count() {
 
 Tiling tiling(const TcNet& N, int most) {
     Tiling T{N.D, N.H, N.W, (N.W + TX - 1) / TX, (N.H + TY - 1) / TY, most, 0};
-    T.planes = (long long)T.tiles_x * T.tiles_y * N.batch * N.D;
+    T.planes = T.tiles_x * T.tiles_y * N.batch * N.D;
     return T;
 }
 
@@ -865,7 +925,7 @@ template <int KC, int NB, int MODE>
 cudaError_t launch_conv(const TcNet& N, ConvArgs A, int* ctas, cudaStream_t s) {
     using Sh = ConvShape<KC, NB>;
     A.t = tiling(N, kMaxPlanes);
-    *ctas = (int)std::min<long long>(A.t.planes, 2 * N.ctas);  // two per SM
+    *ctas = std::min(A.t.planes, 2 * N.ctas);  // two per SM
     cudaError_t e = cudaFuncSetAttribute(conv_tc_kernel<KC, NB, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::kSmem);
     if (e != cudaSuccess) return e;
     conv_tc_kernel<KC, NB, MODE><<<*ctas, kConvThreads, Sh::kSmem, s>>>(A);
@@ -876,7 +936,7 @@ template <int KA, int KB>
 cudaError_t launch_wgrad(const TcNet& N, WgradArgs A, int* ctas, cudaStream_t s) {
     using Sh = WgradShape<KA, KB>;
     A.t = tiling(N, N.D);
-    *ctas = (int)std::min<long long>(A.t.planes, N.ctas);
+    *ctas = std::min(A.t.planes, N.ctas);
     cudaError_t e = cudaFuncSetAttribute(wgrad_tc_kernel<KA, KB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::kSmem);
     if (e != cudaSuccess) return e;
     wgrad_tc_kernel<KA, KB><<<*ctas, kWgThreads, Sh::kSmem, s>>>(A);
