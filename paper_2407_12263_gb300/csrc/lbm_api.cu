@@ -352,38 +352,22 @@ int lbm::ctx_error(lbm_ctx* c, int code, const char* msg) { return set_error(c, 
 
 int lbm::ctx_check(lbm_ctx* c) { return check_ctx(c); }
 
-int lbm::ctx_mass_fixed(lbm_ctx* c, long long* sum) {
-    int rc = check_ctx(c);
-    if (rc) return rc;
-    if (!c->initialised) return set_error(c, LBM_ESTATE, "no state: call lbm_init_phi first");
-    LBM_CUDA(c, lbm::launch_phi_fixed_sum(c->P, c->fg[c->cur], c->partials, c->n_partials, c->result, c->stream));
-    c->launches += 2;
-    double r3;
-    LBM_CUDA(c, cudaMemcpyAsync(&r3, c->result + 3, sizeof r3, cudaMemcpyDeviceToHost, c->stream));
-    LBM_CUDA(c, cudaStreamSynchronize(c->stream));
-    std::memcpy(sum, &r3, sizeof *sum);
-    return LBM_OK;
-}
+void lbm::ctx_drop_graphs(lbm_ctx* c) { drop_graphs(c); }
 
-int lbm::ctx_restart_from_coarse(lbm_ctx* c, int f, const float* coarse, double p0) {
-    int rc = check_ctx(c);
-    if (rc) return rc;
+int lbm::ctx_restart(lbm_ctx* c, int f, const float* coarse, double p0, const long long* before, void* fg, RestartSums* sums) {
     Params& P = c->P;
-    P.w0d = p0 * 3.0;
-    P.w0 = (float)P.w0d;
-    drop_graphs(c);
-    rc = ensure_staging(c, ((size_t)P.N + 1) / 2);  // N floats of upsampled phi
+    const double w0d = p0 * 3.0;
+    if (w0d != P.w0d) {
+        P.w0d = w0d;
+        P.w0 = (float)w0d;
+        drop_graphs(c);  // captured steps carry the old level
+    }
+    int rc = ensure_staging(c, ((size_t)P.N + 1) / 2);  // N floats of upsampled phi
     if (rc) return rc;
-    LBM_CUDA(c, lbm::launch_restart(P, coarse, f, p0, reinterpret_cast<float*>(c->staging), c->fg[c->cur], c->stream));
+    // 8-byte slots in the reduction scratch, enough that blocks rarely meet in one
+    *sums = RestartSums{before, reinterpret_cast<unsigned long long*>(c->partials), std::min(32, 3 * c->n_partials)};
+    LBM_CUDA(c, lbm::launch_restart(P, coarse, f, p0, reinterpret_cast<float*>(c->staging), fg, *sums, c->stream));
     c->launches += 2;
-    c->initialised = true;
-    c->version += 1;
-    return LBM_OK;
-}
-
-int lbm::ctx_adjust_phi(lbm_ctx* c, long long delta) {
-    LBM_CUDA(c, lbm::launch_adjust_phi(c->P, c->fg[c->cur], delta, c->stream));
-    c->launches += 1;
     return LBM_OK;
 }
 

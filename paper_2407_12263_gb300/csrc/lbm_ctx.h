@@ -37,6 +37,8 @@ struct lbm_ctx {
 
 namespace lbm {
 
+struct RestartSums;  // surrogate.h
+
 // lbm_create with the state buffers sized for alloc_storage (>= the bytes of opts->storage), so
 // that set_ctx_storage may later switch to any storage that fits. Messages of a failed create
 // are in lbm_last_error(NULL).
@@ -53,12 +55,11 @@ int set_ctx_storage(lbm_ctx* c, int storage);
 // Helpers of the surrogate entry points (lbm_surrogate.cu).
 int ctx_error(lbm_ctx* c, int code, const char* msg);
 int ctx_check(lbm_ctx* c);
-// The exact 64-bit sum of the fixed-point phi values of the propagated state. Synchronous.
-int ctx_mass_fixed(lbm_ctx* c, long long* sum);
-// Replace the state by the one lbm_init_fields builds from the coarse fields [5][nz/f][ny/f][nx/f]
-// (device FP32: phi, u, v, w, p) upsampled trilinearly; p0 = the storage reference pressure.
-int ctx_restart_from_coarse(lbm_ctx* c, int f, const float* coarse, double p0);
-// Add delta fixed-point units of phi, spread so that the sum changes by exactly delta.
-int ctx_adjust_phi(lbm_ctx* c, long long delta);
+void ctx_drop_graphs(lbm_ctx* c);  // captured steps, after a change of parameters
+// The state lbm_init_fields builds from the coarse fields [5][nz/f][ny/f][nx/f] (device FP32: phi, u,
+// v, w, p) upsampled trilinearly, into the state buffer fg; p0 = the storage reference pressure. *sums
+// is what launch_balance (or launch_coarse_phi) then takes to set sum phi to *before (device).
+// Asynchronous; holds the handle's reduction scratch until then.
+int ctx_restart(lbm_ctx* c, int f, const float* coarse, double p0, const long long* before, void* fg, RestartSums* sums);
 
 }  // namespace lbm

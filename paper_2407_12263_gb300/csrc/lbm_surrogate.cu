@@ -407,7 +407,7 @@ int lbm_coarse_phi(lbm_ctx* c, int f, float* out) {
     if (!out || f < 1 || f > 32 || 32 % f || c->P.nx % f || c->P.ny % f || c->P.nz % f)
         return lbm::ctx_error(c, LBM_EINVAL, "factor must divide 32, nx, ny and nz, and out may not be NULL");
     if (!c->initialised) return lbm::ctx_error(c, LBM_ESTATE, "no state: call lbm_init_phi first");
-    cudaError_t e = lbm::launch_coarse_phi(c->P, c->fg[c->cur], f, out, c->stream);
+    cudaError_t e = lbm::launch_coarse_phi(c->P, c->fg[c->cur], f, nullptr, out, c->stream);
     if (e != cudaSuccess) return lbm::ctx_error(c, LBM_ECUDA, cudaGetErrorString(e));
     c->launches += 1;
     return LBM_OK;
@@ -420,19 +420,18 @@ int lbm_restart_from_coarse(lbm_ctx* c, int f, const float* coarse, double p0) {
         return lbm::ctx_error(c, LBM_EINVAL, "factor must divide nx, ny and nz, and coarse may not be NULL");
     if (!(p0 > 0) || !std::isfinite(p0)) return lbm::ctx_error(c, LBM_EINVAL, "p0 must be > 0 and finite");
     if (!c->initialised) return lbm::ctx_error(c, LBM_ESTATE, "no state to hold the mass of: call lbm_init_phi first");
-    long long before = 0, after = 0;
-    rc = lbm::ctx_mass_fixed(c, &before);
-    if (rc) return rc;
-    rc = lbm::ctx_restart_from_coarse(c, f, coarse, p0);
-    if (rc) return rc;
-    rc = lbm::ctx_mass_fixed(c, &after);
-    if (rc) return rc;
-    if (after != before) {
-        rc = lbm::ctx_adjust_phi(c, before - after);
-        if (rc) return rc;
-    }
-    cudaError_t e = cudaStreamSynchronize(c->stream);
+    // the sum before and the restarted sum stay on the device, where the difference is spread
+    lbm::RestartSums sums;
+    void* fg = c->fg[c->cur];
+    cudaError_t e = lbm::launch_phi_fixed_sum(c->P, fg, c->partials, c->n_partials, c->result, c->stream);
     if (e != cudaSuccess) return lbm::ctx_error(c, LBM_ECUDA, cudaGetErrorString(e));
+    rc = lbm::ctx_restart(c, f, coarse, p0, reinterpret_cast<const long long*>(c->result + 3), fg, &sums);
+    if (rc) return rc;
+    c->version += 1;
+    e = lbm::launch_balance(c->P, fg, sums, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess) return lbm::ctx_error(c, LBM_ECUDA, cudaGetErrorString(e));
+    c->launches += 3;
     return LBM_OK;
 }
 
@@ -445,10 +444,10 @@ bool jump_projects(const lbm_ctx* c, int f) {
     return c->P.walls == 0 && lbm::project_extents_ok(grid_c);
 }
 
-// Carves the jump's buffers out of the handle's workspace, growing it if it is too small: a
-// backup state, four coarse field arrays, the judge's four FP64 measures and the projection's
+// Carves the jump's buffers out of the handle's workspace, growing it if it is too small: a third
+// state buffer, four coarse field arrays, the judge's measures (Measure) and the projection's
 // scratch (*proj, NULL when the jump does not project).
-int jump_workspace(lbm_ctx* c, int f, void** backup, float* fields[4], double** measures, void** proj) {
+int jump_workspace(lbm_ctx* c, int f, void** third, float* fields[4], double** measures, void** proj) {
     const long long nc = (long long)(c->P.nx / f) * (c->P.ny / f) * (c->P.nz / f);
     const size_t align = 256;
     const size_t sb = (c->fg_bytes + align - 1) / align * align;
@@ -464,12 +463,16 @@ int jump_workspace(lbm_ctx* c, int f, void** backup, float* fields[4], double** 
         c->jump_ws_bytes = need;
     }
     char* base = static_cast<char*>(c->jump_ws);
-    *backup = base;
+    *third = base;
     for (int i = 0; i < 4; ++i) fields[i] = reinterpret_cast<float*>(base + sb + i * fb);
     *measures = reinterpret_cast<double*>(base + sb + 4 * fb);
     *proj = pb ? base + sb + 4 * fb + align : nullptr;
     return LBM_OK;
 }
+
+// The device doubles of a jump: four of launch_jump_measures, the fixed-point sum of phi before it
+// (integer bits), a tensor-core timeout (integer bits) and the two relaxation rates (times steps).
+enum Measure { kPredSum, kShift, kGrad, kSpeed2, kSumBefore, kTimeout, kRateRef, kRatePred, kMeasures };
 
 }  // namespace
 
@@ -478,11 +481,11 @@ int lbm_surrogate_reserve(lbm_ctx* c, int f) {
     if (rc) return rc;
     if (f < 1 || c->P.nx % f || c->P.ny % f || c->P.nz % f)
         return lbm::ctx_error(c, LBM_EINVAL, "factor must divide nx, ny and nz");
-    void* backup;
+    void* third;
     float* fields[4];
     double* measures;
     void* proj;
-    return jump_workspace(c, f, &backup, fields, &measures, &proj);
+    return jump_workspace(c, f, &third, fields, &measures, &proj);
 }
 
 int lbm_surrogate_jump(lbm_ctx* c, lbm_net* n, int f, const float mean_std[10], int k, int judge_steps, double mass_tol,
@@ -499,26 +502,28 @@ int lbm_surrogate_jump(lbm_ctx* c, lbm_net* n, int f, const float mean_std[10], 
     std::memset(rep, 0, sizeof *rep);
     const int grid_c[3] = {c->P.nx / f, c->P.ny / f, c->P.nz / f};
     const long long nc = (long long)grid_c[0] * grid_c[1] * grid_c[2];
-    void* backup;
+    void* third;
     float* fields[4];
     double* measures;
     void* proj;
-    if ((rc = jump_workspace(c, f, &backup, fields, &measures, &proj))) return rc;
+    if ((rc = jump_workspace(c, f, &third, fields, &measures, &proj))) return rc;
     float *in = fields[0], *xin = fields[1], *yout = fields[2], *pred = fields[3];
     auto cu = [&](cudaError_t e) { return e == cudaSuccess ? LBM_OK : lbm::ctx_error(c, LBM_ECUDA, cudaGetErrorString(e)); };
-    const int saved_cur = c->cur;
     const lbm::Params saved_P = c->P;
-    if ((rc = cu(cudaMemcpyAsync(backup, c->fg[c->cur], c->fg_bytes, cudaMemcpyDeviceToDevice, c->stream)))) return rc;
-    long long m_before = 0;
-    if ((rc = lbm::ctx_mass_fixed(c, &m_before))) return rc;
+    void* const start = c->fg[c->cur];  // read, never written, until the jump is accepted
+    if ((rc = cu(cudaMemsetAsync(measures, 0, kMeasures * sizeof(double), c->stream)))) return rc;
+    // sum phi before, in place 3 of the four results
+    if ((rc = cu(lbm::launch_phi_fixed_sum(c->P, start, c->partials, c->n_partials, measures + kSumBefore - 3, c->stream)))) return rc;
+    c->launches += 2;
     // 1. predict
     if ((rc = lbm_coarse_fields(c, f, in))) return rc;
-    if ((rc = cu(cudaStreamSynchronize(c->stream)))) return rc;
+    const bool apart = n->stream != c->stream;
+    if (apart && (rc = cu(cudaStreamSynchronize(c->stream)))) return rc;
     if ((rc = cu(lbm::launch_normalize(in, xin, nc, mean_std, +1, n->stream)))) return rc;
     if ((rc = lbm_net_forward(n, xin, yout, 1, grid_c))) return lbm::ctx_error(c, rc, lbm_net_last_error(n));
     if ((rc = cu(lbm::launch_normalize(yout, pred, nc, mean_std, -1, n->stream)))) return rc;
-    if ((rc = cu(cudaStreamSynchronize(n->stream)))) return rc;
-    if ((rc = check_tc(n))) return lbm::ctx_error(c, rc, lbm_net_last_error(n));
+    if (apart && (rc = cu(cudaStreamSynchronize(n->stream)))) return rc;
+    if ((rc = cu(cudaMemcpyAsync(measures + kTimeout, n->tc_err, sizeof(int), cudaMemcpyDeviceToDevice, c->stream)))) return rc;
     // the predicted velocity (channels 1-3) replaced by its divergence-free part
     if (proj) {
         if ((rc = cu(lbm::launch_project_solenoidal(pred + nc, grid_c[0], grid_c[1], grid_c[2], proj, c->stream))))
@@ -527,64 +532,78 @@ int lbm_surrogate_jump(lbm_ctx* c, lbm_net* n, int f, const float mean_std[10], 
         rep->projected = 1;
     }
     // 2. mass and interface position of the prediction, measured on the coarse grid
-    if ((rc = cu(cudaMemsetAsync(measures, 0, 4 * sizeof(double), c->stream)))) return rc;
     if ((rc = cu(lbm::launch_jump_measures(in, pred, grid_c[0], grid_c[1], grid_c[2], c->P.walls, measures, c->stream))))
         return rc;
-    double m[4];
+    double m[kMeasures];
     if ((rc = cu(cudaMemcpyAsync(m, measures, sizeof m, cudaMemcpyDeviceToHost, c->stream)))) return rc;
     if ((rc = cu(cudaStreamSynchronize(c->stream)))) return rc;
     c->launches += 1;
+    int timeout;
+    std::memcpy(&timeout, &m[kTimeout], sizeof timeout);
+    if (timeout && (rc = check_tc(n))) return lbm::ctx_error(c, rc, lbm_net_last_error(n));
+    long long m_before;
+    std::memcpy(&m_before, &m[kSumBefore], sizeof m_before);
     const double mass_before = (double)m_before / 1073741824.0;
-    const double mass_pred = m[0] * f * f * f, jump = m[1];
+    const double mass_pred = m[kPredSum] * f * f * f, jump = m[kShift];
     rep->mass_error = std::fabs(mass_pred - mass_before) / std::fabs(mass_before);
     // Mean displacement of the interface, in fine cells: a profile moved by d along its normal
     // changes phi by |grad phi| d, so int |phi_pred - phi_start| dV = d int |grad phi| dV. On the
     // coarse grid both integrals are sums over coarse cells (f^3 fine cells each; the coarse
     // gradient is f times the fine one), so d = f sum |dphi| / sum |grad_c phi|.
-    rep->interface_shift = m[2] > 0 ? f * jump / m[2] : (jump > 0 ? INFINITY : 0.0);
+    rep->interface_shift = m[kGrad] > 0 ? f * jump / m[kGrad] : (jump > 0 ? INFINITY : 0.0);
     // Kinematic bound: the phi = 1/2 surface is carried by the flow (the sharpening flux of the
     // conservative phase-field equation vanishes on the equilibrium profile), so in k steps no
     // part of it moves farther than the largest speed times k.
-    rep->interface_limit = interface_tol * std::sqrt(m[3]) * k;
+    rep->interface_limit = interface_tol * std::sqrt(m[kSpeed2]) * k;
     bool accept = rep->mass_error <= mass_tol && rep->interface_shift <= rep->interface_limit;
     // 3-4. restart and judge. How fast phi moves in the LBM's first judge_steps steps after a
     // restart, as the L1 rate of its coarse block means: after the restart from the prediction,
     // against the same after the restart from the starting state's own coarse fields. Both carry
     // the relaxation a restart causes (upsampled fields are smoother than the lattice's); a
     // prediction whose phi, u and p do not fit together relaxes faster than that.
+    // The restarts and their steps run in the handle's other buffer and the third one, ending in the
+    // former, and everything stays on the device until both rates are known; the starting state is
+    // neither copied nor touched.
     if (accept) {
-        auto coarse_phi_into = [&](float* dst) -> int {
-            if (f <= 32 && 32 % f == 0) return cu(lbm::launch_coarse_phi(c->P, c->fg[c->cur], f, dst, c->stream));
-            return lbm_coarse_fields(c, f, dst);  // phi is channel 0 of the five it writes
-        };
-        std::vector<float> h_r((size_t)nc), h_after((size_t)nc);
+        void* const other = c->fg[1 - c->cur];
+        const bool phi_blocks = f <= 32 && 32 % f == 0;
         auto restart_and_relax = [&](const float* src, double* rate) -> int {
-            int r = lbm_restart_from_coarse(c, f, src, saved_P.w0d / 3.0);
+            void* from = judge_steps % 2 ? third : other;
+            void* to = judge_steps % 2 ? other : third;
+            lbm::RestartSums sums;
+            int r = lbm::ctx_restart(c, f, src, saved_P.w0d / 3.0, reinterpret_cast<const long long*>(measures + kSumBefore), from, &sums);
             if (r) return r;
-            if ((r = coarse_phi_into(xin))) return r;
-            if ((r = lbm_step(c, judge_steps))) return r;
-            if ((r = coarse_phi_into(yout))) return r;
-            if ((r = cu(cudaStreamSynchronize(c->stream)))) return r;
-            if ((r = cu(cudaMemcpy(h_r.data(), xin, (size_t)nc * sizeof(float), cudaMemcpyDeviceToHost)))) return r;
-            if ((r = cu(cudaMemcpy(h_after.data(), yout, (size_t)nc * sizeof(float), cudaMemcpyDeviceToHost)))) return r;
-            double sum = 0.0;
-            for (long long i = 0; i < nc; ++i) sum += std::fabs((double)h_after[i] - (double)h_r[i]);
-            *rate = sum / judge_steps;
-            return LBM_OK;
+            if (phi_blocks) {
+                if ((r = cu(lbm::launch_coarse_phi(c->P, from, f, &sums, xin, c->stream)))) return r;
+            } else {  // phi is channel 0 of the five fields
+                if ((r = cu(lbm::launch_balance(c->P, from, sums, c->stream)))) return r;
+                if ((r = cu(lbm::launch_coarsen(c->P, from, f, xin, c->stream)))) return r;
+            }
+            for (int j = 0; j < judge_steps; ++j, std::swap(from, to)) {
+                int launches = 0;
+                if ((r = cu(lbm::launch_step(c->P, lbm::SCHEME_DF, from, to, nullptr, c->stream, &launches)))) return r;
+                c->launches += launches;
+            }
+            r = cu(phi_blocks ? lbm::launch_coarse_phi(c->P, from, f, nullptr, yout, c->stream)
+                              : lbm::launch_coarsen(c->P, from, f, yout, c->stream));
+            if (r) return r;
+            c->launches += phi_blocks ? 4 : 5;
+            return cu(lbm::launch_l1_difference(xin, yout, nc, c->partials, 3 * c->n_partials, rate, c->stream));
         };
-        double rate_ref = 0.0, rate_pred = 0.0;
-        if ((rc = restart_and_relax(in, &rate_ref))) return rc;
-        if ((rc = restart_and_relax(pred, &rate_pred))) return rc;
+        if ((rc = restart_and_relax(in, measures + kRateRef))) return rc;
+        if ((rc = restart_and_relax(pred, measures + kRatePred))) return rc;
+        if ((rc = cu(cudaMemcpyAsync(m, measures, sizeof m, cudaMemcpyDeviceToHost, c->stream)))) return rc;
+        if ((rc = cu(cudaStreamSynchronize(c->stream)))) return rc;
+        const double rate_ref = m[kRateRef] / judge_steps, rate_pred = m[kRatePred] / judge_steps;
         rep->relax_ratio = rate_ref > 0 ? rate_pred / rate_ref : (rate_pred > 0 ? INFINITY : 0.0);
         accept = rep->relax_ratio <= relax_tol;
     }
-    // 5. fallback
-    if (!accept) {
+    c->version += 1;
+    if (accept) {
+        c->cur = 1 - c->cur;
+    } else {  // 5. fallback
+        if (c->P.w0d != saved_P.w0d) lbm::ctx_drop_graphs(c);
         c->P = saved_P;
-        c->cur = saved_cur;
-        if ((rc = cu(cudaMemcpyAsync(c->fg[c->cur], backup, c->fg_bytes, cudaMemcpyDeviceToDevice, c->stream)))) return rc;
-        c->initialised = true;
-        c->version += 1;
         if ((rc = lbm_step(c, k))) return rc;
         if ((rc = cu(cudaStreamSynchronize(c->stream)))) return rc;
     }

@@ -74,17 +74,29 @@ cudaError_t tc_run(const TcNet& N, const float* x, float* y, const float* target
 // Coarse fields [5][nz/f][ny/f][nx/f] (phi, u, v, w, p; means over f^3 cells of the macroscopic
 // fields of the difference-free scheme) of the propagated state fg.
 cudaError_t launch_coarsen(const Params& P, const void* fg, int factor, float* out, cudaStream_t s);
+// Device sums around a restart: *before is the fixed-point sum of phi that the state must keep,
+// slots[0 .. n_slots) receive the restarted state's (their total).
+struct RestartSums {
+    const long long* before;
+    unsigned long long* slots;
+    int n_slots;
+};
 // Block means of the state's own phi (plane 0, before propagation) into out [nz/f][ny/f][nx/f];
-// factor must divide 32 (cudaErrorInvalidValue otherwise).
-cudaError_t launch_coarse_phi(const Params& P, const void* fg, int factor, float* out, cudaStream_t s);
+// factor must divide 32 (cudaErrorInvalidValue otherwise). With sums the state is balanced first
+// (launch_balance), in the same pass.
+cudaError_t launch_coarse_phi(const Params& P, void* fg, int factor, const RestartSums* sums, float* out, cudaStream_t s);
 // The state launch_init builds (equilibrium plus the first-order non-equilibrium part of g) from
 // coarse fields upsampled trilinearly between coarse cell centres (periodic, clamped across
 // walls), in FP32 arithmetic: the upsampled phi of every cell into phi_fine (N floats), then the
-// populations.
+// populations and sums.slots.
 cudaError_t launch_restart(const Params& P, const float* coarse, int factor, double p0, float* phi_fine, void* fg,
-                           cudaStream_t s);
-// Adds delta units (2^-30) of phi to the state, spread over the cells so that it sums exactly.
-cudaError_t launch_adjust_phi(const Params& P, void* fg, long long delta, cudaStream_t s);
+                           const RestartSums& sums, cudaStream_t s);
+// Adds *before minus the slots' total, in units (2^-30) of phi, spread over the cells of the state so
+// that its sum is *before exactly.
+cudaError_t launch_balance(const Params& P, void* fg, const RestartSums& sums, cudaStream_t s);
+// *out = sum |a - b| over n values, FP64 in a fixed order; partials: n_partials doubles of scratch.
+cudaError_t launch_l1_difference(const float* a, const float* b, long long n, double* partials, int n_partials, double* out,
+                                 cudaStream_t s);
 // What the judge of a jump measures on the coarse grid [5][ncz][ncy][ncx] of the starting fields
 // `start` and of the prediction `pred`, accumulated into out[4] (zeroed by the caller):
 //   out[0] += sum of the predicted phi;

@@ -2,6 +2,8 @@
 // block means of the macroscopic fields, the restart from trilinearly upsampled coarse fields
 // (the same equilibrium-plus-non-equilibrium construction as the initial state, in FP32), and
 // the exact correction of sum phi after a restart.
+#include <algorithm>
+
 #include "cell.cuh"
 #include "surrogate.h"
 
@@ -309,31 +311,112 @@ cudaError_t launch_coarsen(const Params& P, const void* fg, int factor, float* o
     return cudaGetLastError();
 }
 
-// Block means over f^3 cells of the state's own phi, the fixed-point value of plane 0 (no
-// propagation: 8 bytes read per cell). Lane l of a warp takes fine x = 32 b + l; f divides 32,
-// and each aligned group of f lanes is summed with shuffles.
-__global__ void coarse_phi_kernel(const float2* __restrict__ plane0, int nx, int ny, int nz, int f, float* __restrict__ out) {
+// What the sum of a restarted state's fixed-point phi must be raised by, cell by cell: every cell by
+// q and the first |r| cells by the sign of r more, q N + r = before - the sum of the slots (the sums of
+// the restarted blocks). Read by one thread of a block; the others take it from shared memory.
+struct Balance {
+    const long long* before;  // NULL: nothing to add
+    const unsigned long long* slots;
+    int n_slots;
+    long long N;
+};
+__device__ __forceinline__ void balance_of(const Balance& B, long long (&s_qr)[2]) {
+    if (threadIdx.x == 0 && threadIdx.y == 0) {
+        unsigned long long after = 0;
+        for (int i = 0; i < B.n_slots; ++i) after += B.slots[i];
+        const long long delta = *B.before - (long long)after;
+        s_qr[0] = delta / B.N;
+        s_qr[1] = delta - s_qr[0] * B.N;
+    }
+    __syncthreads();
+}
+__device__ __forceinline__ int balanced(int phi_fx, long long c, const long long (&qr)[2]) {
+    const long long ar = qr[1] < 0 ? -qr[1] : qr[1];
+    const long long add = qr[0] + (c < ar ? (qr[1] < 0 ? -1 : 1) : 0);
+    return (int)((unsigned int)phi_fx + (unsigned int)add);
+}
+
+// Block means over F^3 cells of the state's own phi, the fixed-point value of plane 0 (no
+// propagation: 8 bytes read per cell), after the balance has been added and stored, if there is one.
+// Lane l of a warp takes fine x = 32 b + l; F divides 32, and each aligned group of F lanes is summed
+// with shuffles. With the factor known the loads of eight rows are in flight at once: 128^3 at F = 2
+// 18 -> 6 us, 9 us with the balance (8.6 us as a pass of its own).
+template <int F, bool BALANCE>
+__global__ void __launch_bounds__(128) coarse_phi_kernel(float2* __restrict__ plane0, int nx, int ny, int nz, const Balance B,
+                                                         float* __restrict__ out) {
+    __shared__ long long s_qr[2];
+    if (BALANCE) balance_of(B, s_qr);
     const int lane = threadIdx.x;
     const int x = blockIdx.x * 32 + lane;
     const int cy = blockIdx.y * blockDim.y + threadIdx.y;
     const int cz = blockIdx.z;
-    const int ncx = nx / f, ncy = ny / f;
+    const int ncx = nx / F, ncy = ny / F;
     if (cy >= ncy) return;  // whole warps leave together
     const bool valid = x < nx;
+    constexpr int kRows = F * F, kStep = kRows < 8 ? kRows : 8;
     long long acc = 0;
     if (valid)
-        for (int dz = 0; dz < f; ++dz)
-            for (int dy = 0; dy < f; ++dy)
-                acc += __float_as_int(__ldg(plane0 + ((long long)(cz * f + dz) * ny + (cy * f + dy)) * nx + x).y);
-    for (int o = f >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (!valid || lane % f) return;
-    out[((long long)cz * ncy + cy) * ncx + x / f] = (float)((double)acc / (kPhiFx * (double)f * f * f));
+        for (int r0 = 0; r0 < kRows; r0 += kStep) {
+            long long c[kStep];
+            int v[kStep];
+#pragma unroll
+            for (int k = 0; k < kStep; ++k) {
+                const int r = r0 + k;
+                c[k] = ((long long)(cz * F + r / F) * ny + (cy * F + r % F)) * nx + x;
+                v[k] = __float_as_int(plane0[c[k]].y);
+            }
+#pragma unroll
+            for (int k = 0; k < kStep; ++k) {
+                if (BALANCE) {
+                    v[k] = balanced(v[k], c[k], s_qr);
+                    plane0[c[k]].y = __int_as_float(v[k]);
+                }
+                acc += v[k];
+            }
+        }
+#pragma unroll
+    for (int o = F >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (!valid || lane % F) return;
+    out[((long long)cz * ncy + cy) * ncx + x / F] = (float)((double)acc / (kPhiFx * (double)F * F * F));
 }
 
-cudaError_t launch_coarse_phi(const Params& P, const void* fg, int factor, float* out, cudaStream_t s) {
-    if (factor > 32 || 32 % factor) return cudaErrorInvalidValue;
-    const dim3 block(32, 4), grid((P.nx + 31) / 32, (P.ny / factor + 3) / 4, P.nz / factor);
-    coarse_phi_kernel<<<grid, block, 0, s>>>(moment_plane(fg), P.nx, P.ny, P.nz, factor, out);
+__global__ void balance_kernel(float2* __restrict__ plane0, const Balance B) {
+    __shared__ long long s_qr[2];
+    balance_of(B, s_qr);
+    if (s_qr[0] == 0 && s_qr[1] == 0) return;
+    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < B.N; c += (long long)gridDim.x * blockDim.x)
+        plane0[c].y = __int_as_float(balanced(__float_as_int(plane0[c].y), c, s_qr));
+}
+
+static unsigned cell_blocks(long long n) { return (unsigned)std::min<long long>((n + 255) / 256, 4096); }
+
+static Balance balance_of_restart(const Params& P, const RestartSums* sums) {
+    return sums ? Balance{sums->before, sums->slots, sums->n_slots, P.N} : Balance{nullptr, nullptr, 0, P.N};
+}
+
+cudaError_t launch_balance(const Params& P, void* fg, const RestartSums& sums, cudaStream_t s) {
+    balance_kernel<<<cell_blocks(P.N), 256, 0, s>>>(moment_plane(fg), balance_of_restart(P, &sums));
+    return cudaGetLastError();
+}
+
+template <int F>
+static void coarse_phi_f(const Params& P, void* fg, const RestartSums* sums, float* out, cudaStream_t s) {
+    const dim3 block(32, 4), grid((P.nx + 31) / 32, (P.ny / F + 3) / 4, P.nz / F);
+    const Balance B = balance_of_restart(P, sums);
+    if (sums) coarse_phi_kernel<F, true><<<grid, block, 0, s>>>(moment_plane(fg), P.nx, P.ny, P.nz, B, out);
+    else coarse_phi_kernel<F, false><<<grid, block, 0, s>>>(moment_plane(fg), P.nx, P.ny, P.nz, B, out);
+}
+
+cudaError_t launch_coarse_phi(const Params& P, void* fg, int factor, const RestartSums* sums, float* out, cudaStream_t s) {
+    switch (factor) {
+        case 1: coarse_phi_f<1>(P, fg, sums, out, s); break;
+        case 2: coarse_phi_f<2>(P, fg, sums, out, s); break;
+        case 4: coarse_phi_f<4>(P, fg, sums, out, s); break;
+        case 8: coarse_phi_f<8>(P, fg, sums, out, s); break;
+        case 16: coarse_phi_f<16>(P, fg, sums, out, s); break;
+        case 32: coarse_phi_f<32>(P, fg, sums, out, s); break;
+        default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
 }
 
@@ -401,12 +484,8 @@ __device__ __forceinline__ float trilinear(const float* __restrict__ q, const Co
     return lerp(lerp(c00, c01, c.ty), lerp(c10, c11, c.ty), c.tz);
 }
 
-// The initial-state construction of init_kernel (equilibria of the upsampled phi, u, p plus the
-// first-order non-equilibrium part of g, grad phi from the isotropic central difference of the
-// upsampled phi, which phi_fine_kernel writes first) in FP32, written directly as deviations
-// from the storage's reference levels. phi is clamped to [-1, 1.5], the range lbm_init_fields
-// accepts, so that its fixed-point value stays in range whatever the prediction holds.
-// The upsampled phi of every cell (clamped as below), the first pass of the restart.
+// The upsampled phi of every cell, the first pass of the restart, clamped to [-1, 1.5], the range
+// lbm_init_fields accepts, so that its fixed-point value stays in range whatever the prediction holds.
 __global__ void phi_fine_kernel(const Params P, const float* __restrict__ coarse, int f, float* __restrict__ phi) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -418,34 +497,27 @@ __global__ void phi_fine_kernel(const Params P, const float* __restrict__ coarse
     phi[((long long)z * P.ny + y) * P.nx + x] = fminf(fmaxf(v, -1.0f), 1.5f);
 }
 
+// The second: the initial-state construction of init_kernel (equilibria of the upsampled phi, u, p plus
+// the first-order non-equilibrium part of g, grad phi from the isotropic central difference of the
+// upsampled phi) in FP32, directly as deviations from the storage's reference levels. The words of
+// opposite pairs are stored whole (a store per population writes half of every sector it touches), and
+// the block's sum of the fixed-point phi goes to one of the slots (integer atomics: the same total in
+// any order). Bound by instructions: the arithmetic is written with the velocities' zero components,
+// and 16-bit restarts, which amplify a last bit, fix its roundings.
 template <int Q, int S>
-__global__ void restart_kernel(const Params P, const float* __restrict__ coarse, const float* __restrict__ phi_fine, int f,
-                               float p0, void* __restrict__ fg) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    if (x >= P.nx || y >= P.ny) return;
+__device__ __forceinline__ int restart_cell(const Params& P, const float* __restrict__ coarse, const float* __restrict__ phi_fine,
+                                            int f, float p0, void* __restrict__ fg, int x, int y, int z) {
     const int ncx = P.nx / f, ncy = P.ny / f, ncz = P.nz / f;
     const long long nc = (long long)ncx * ncy * ncz;
-    // neighbour rows and columns: periodic images, or across a wall the cell itself (so that
-    // the normal gradient vanishes there)
-    int xs[3], ys[3], zs[3];
-    // x + d lies in [-1, nx]: a periodic image is one period away at most
-    auto wrap1 = [](int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); };
-#pragma unroll
-    for (int d = -1; d <= 1; ++d) {
-        xs[d + 1] = (P.walls & 1) ? min(max(x + d, 0), P.nx - 1) : wrap1(x + d, P.nx);
-        ys[d + 1] = (P.walls & 2) ? min(max(y + d, 0), P.ny - 1) : wrap1(y + d, P.ny);
-        zs[d + 1] = (P.walls & 4) ? min(max(z + d, 0), P.nz - 1) : wrap1(z + d, P.nz);
-    }
-    auto phi_at = [&](int dx, int dy, int dz) {  // the grid holds fewer than 2^31 cells
-        return __ldg(phi_fine + (zs[dz + 1] * P.ny + ys[dy + 1]) * P.nx + xs[dx + 1]);
-    };
-    const float phi = phi_at(0, 0, 0);
+    // neighbours: periodic images, or across a wall the cell itself (so that the normal gradient
+    // vanishes there); the grid holds fewer than 2^31 cells
+    const Nbr nb = mirror_at_walls(make_nbr(P, x, y, z), make_wall_side(P, x, y, z));
+    const float* __restrict__ here = phi_fine + ((z * P.ny + y) * P.nx + x);
+    const float phi = __ldg(here);
     float gx = 0.f, gy = 0.f, gz = 0.f;
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
-        const float v = Lat<Q>::w(i) * phi_at(Lat<Q>::cx(i), Lat<Q>::cy(i), Lat<Q>::cz(i));
+        const float v = Lat<Q>::w(i) * __ldg(here + link_offset<Q>(nb, i, +1));
         gx += Lat<Q>::cx(i) * v;
         gy += Lat<Q>::cy(i) * v;
         gz += Lat<Q>::cz(i) * v;
@@ -471,7 +543,7 @@ __global__ void restart_kernel(const Params P, const float* __restrict__ coarse,
     const float Phi = phi - P.phi_ref;
     const float tnq = P.tau_phi - 0.5f;
     const long long c = ((long long)z * P.ny + y) * P.nx + x;
-    float fsum = 0.f;
+    float fsum = 0.f, fs[Q], gs[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         const float t = Lat<Q>::w(i);
@@ -484,17 +556,47 @@ __global__ void restart_kernel(const Params P, const float* __restrict__ coarse,
         const float fdev = t * (dP + rho * gam - 4.5f * pis);                        // f*_i - t_i w0
         const float gdev = t * (Phi + phi * gam + P.tau_phi * es) - t * tnq * eg;  // g*_i - t_i phi_ref
         fsum += fdev;
-        if (i > 0) Store<S>::store(pop_ptr<Q, S>(fg, P.N, i, c), fdev, gdev, P);
+        fs[i] = fdev * Store<S>::kScaleF;
+        gs[i] = gdev * Store<S>::kScaleG;
+    }
+#pragma unroll
+    for (int k = 0; k < Lat<Q>::kPairs; ++k) {
+        const int i = Lat<Q>::pair_first(k), j = Lat<Q>::pair_second(k);
+        __stcs(pair_plane<S>(fg, P.N, k) + c, Store<S>::word(fs[i], gs[i], fs[j], gs[j]));
     }
     // plane 0: sum_i f*_i - w0, and phi (= sum_i g*_i) as the integer phi * 2^30
-    moment_plane(fg)[c] = make_float2(fsum, __int_as_float(__float2int_rn(phi * 1073741824.0f)));
+    const int phi_fx = __float2int_rn(phi * 1073741824.0f);
+    moment_plane(fg)[c] = make_float2(fsum, __int_as_float(phi_fx));
+    return phi_fx;
+}
+
+template <int Q, int S>
+__global__ void __launch_bounds__(128)
+restart_kernel(const Params P, const float* __restrict__ coarse, const float* __restrict__ phi_fine, int f, float p0,
+               void* __restrict__ fg, unsigned long long* __restrict__ slots, int n_slots) {
+    __shared__ long long s_sum[4];
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    int v = 0;
+    if (x < P.nx && y < P.ny) v = restart_cell<Q, S>(P, coarse, phi_fine, f, p0, fg, x, y, blockIdx.z);
+    // a warp's sum by halves that cannot overflow
+    const long long sum = ((long long)__reduce_add_sync(0xffffffffu, v >> 16) << 16) +
+                          (long long)__reduce_add_sync(0xffffffffu, (unsigned)v & 0xffffu);
+    if (threadIdx.x == 0) s_sum[threadIdx.y] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0 && threadIdx.y == 0) {
+        const unsigned block = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+        atomicAdd(slots + block % (unsigned)n_slots, (unsigned long long)(s_sum[0] + s_sum[1] + s_sum[2] + s_sum[3]));
+    }
 }
 
 cudaError_t launch_restart(const Params& P, const float* coarse, int factor, double p0, float* phi_fine, void* fg,
-                           cudaStream_t s) {
+                           const RestartSums& sums, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(sums.slots, 0, sums.n_slots * sizeof(*sums.slots), s);
+    if (e != cudaSuccess) return e;
     const dim3 block(32, 4), grid((P.nx + 31) / 32, (P.ny + 3) / 4, P.nz);
     phi_fine_kernel<<<grid, block, 0, s>>>(P, coarse, factor, phi_fine);
-#define LBM_RESTART(Q, S) restart_kernel<Q, S><<<grid, block, 0, s>>>(P, coarse, phi_fine, factor, (float)p0, fg)
+#define LBM_RESTART(Q, S) restart_kernel<Q, S><<<grid, block, 0, s>>>(P, coarse, phi_fine, factor, (float)p0, fg, sums.slots, sums.n_slots)
     if (P.Q == 9) {
         if (P.storage == STORE_F16) LBM_RESTART(9, STORE_F16);
         else if (P.storage == STORE_BF16) LBM_RESTART(9, STORE_BF16);
@@ -505,22 +607,6 @@ cudaError_t launch_restart(const Params& P, const float* coarse, int factor, dou
         else LBM_RESTART(19, STORE_F32);
     }
 #undef LBM_RESTART
-    return cudaGetLastError();
-}
-
-__global__ void adjust_phi_kernel(float2* __restrict__ plane0, long long N, long long q, long long r) {
-    const long long sign = r < 0 ? -1 : 1, ar = r < 0 ? -r : r;
-    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
-        const long long add = q + (c < ar ? sign : 0);
-        const int v = __float_as_int(plane0[c].y);
-        plane0[c].y = __int_as_float((int)((unsigned int)v + (unsigned int)add));
-    }
-}
-
-cudaError_t launch_adjust_phi(const Params& P, void* fg, long long delta, cudaStream_t s) {
-    const long long q = delta / P.N, r = delta - q * P.N;
-    const long long blocks = (P.N + 255) / 256;
-    adjust_phi_kernel<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(moment_plane(fg), P.N, q, r);
     return cudaGetLastError();
 }
 
@@ -603,16 +689,55 @@ cudaError_t launch_jump_measures(const float* start, const float* pred, int ncx,
 __global__ void normalize_kernel(const float* __restrict__ x, float* __restrict__ y, long long n, float m0, float m1,
                                  float m2, float m3, float m4, float s0, float s1, float s2, float s3, float s4, int dir) {
     const float mean[5] = {m0, m1, m2, m3, m4}, sd[5] = {s0, s1, s2, s3, s4};
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < 5 * n; i += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(i / n);
-        y[i] = dir > 0 ? (x[i] - mean[c]) / sd[c] : x[i] * sd[c] + mean[c];
-    }
+    const int c = blockIdx.y;
+    const float m = mean[c], d = sd[c];
+    x += c * n;
+    y += c * n;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        y[i] = dir > 0 ? (x[i] - m) / d : x[i] * d + m;
 }
 
 cudaError_t launch_normalize(const float* x, float* y, long long n, const float* ms, int dir, cudaStream_t s) {
-    const long long blocks = (5 * n + 255) / 256;
-    normalize_kernel<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, s>>>(x, y, n, ms[0], ms[1], ms[2], ms[3], ms[4],
-                                                                              ms[5], ms[6], ms[7], ms[8], ms[9], dir);
+    normalize_kernel<<<dim3(cell_blocks(n), 5), 256, 0, s>>>(x, y, n, ms[0], ms[1], ms[2], ms[3], ms[4], ms[5], ms[6], ms[7],
+                                                            ms[8], ms[9], dir);
+    return cudaGetLastError();
+}
+
+// sum |a - b| over n values in FP64: per block, then the blocks by one block, each in a fixed order.
+__global__ void __launch_bounds__(kJumpThreads) l1_kernel(const float* __restrict__ a, const float* __restrict__ b, long long n,
+                                                         double* __restrict__ out) {
+    __shared__ double red[kJumpThreads / 32];
+    double acc = 0.0;
+    for (long long i = (long long)blockIdx.x * kJumpThreads + threadIdx.x; i < n; i += (long long)gridDim.x * kJumpThreads)
+        acc += fabs((double)__ldg(a + i) - (double)__ldg(b + i));
+    acc = warp_sum_jm(acc);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        acc = 0.0;
+        for (int w = 0; w < kJumpThreads / 32; ++w) acc += red[w];
+        out[blockIdx.x] = acc;
+    }
+}
+__global__ void __launch_bounds__(kJumpThreads) l1_finish(const double* __restrict__ part, int n, double* __restrict__ out) {
+    __shared__ double red[kJumpThreads / 32];
+    double acc = 0.0;
+    for (int i = threadIdx.x; i < n; i += kJumpThreads) acc += part[i];
+    acc = warp_sum_jm(acc);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        acc = 0.0;
+        for (int w = 0; w < kJumpThreads / 32; ++w) acc += red[w];
+        *out = acc;
+    }
+}
+
+cudaError_t launch_l1_difference(const float* a, const float* b, long long n, double* partials, int n_partials, double* out,
+                                 cudaStream_t s) {
+    const int blocks = (int)std::min<long long>((n + kJumpThreads - 1) / kJumpThreads, std::min(n_partials, 512));
+    l1_kernel<<<blocks, kJumpThreads, 0, s>>>(a, b, n, partials);
+    l1_finish<<<1, kJumpThreads, 0, s>>>(partials, blocks, out);
     return cudaGetLastError();
 }
 
