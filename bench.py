@@ -64,7 +64,7 @@ BYTES_PER_CELL_16 = 2 * (8 + 18 * 4)
 PROFILE = ROOT / "profiles" / "step_kernel_droplet3d_128.md"
 KERNEL_SOURCES = ["paper_2407_12263_gb300/csrc/cell.cuh", "paper_2407_12263_gb300/csrc/lattice.cuh",
                   "paper_2407_12263_gb300/csrc/step_kernels.cu", "paper_2407_12263_gb300/csrc/lbm_internal.h",
-                  "paper_2407_12263_gb300/csrc/storage.cuh"]
+                  "paper_2407_12263_gb300/csrc/storage.cuh", "paper_2407_12263_gb300/csrc/chain.cuh"]
 
 
 # ---------------------------------------------------------------- multi-rank helpers (host logic)

@@ -26,6 +26,7 @@ constexpr int batch_min_blocks() {
 template <int Q, bool GEN, int S>
 __global__ void __launch_bounds__(kBatchThreads, (batch_min_blocks<GEN, S>()))
 batch_step_kernel(const __grid_constant__ BatchLaunch L) {
+    chain_begin();
     const LaunchCase& C = L.cases[blockIdx.y];
     // The host groups cases that share every parameter except their fluid properties (see
     // group_key in lbm_batch.cu), so those shared fields are read from case 0, at fixed offsets
@@ -53,24 +54,19 @@ batch_step_kernel(const __grid_constant__ BatchLaunch L) {
 }
 
 template <int Q>
-static void launch_q(const BatchLaunch& L, dim3 grid, cudaStream_t s) {
-    if (L.general) {
-        if (L.storage == STORE_F16) batch_step_kernel<Q, true, STORE_F16><<<grid, kBatchThreads, 0, s>>>(L);
-        else if (L.storage == STORE_BF16) batch_step_kernel<Q, true, STORE_BF16><<<grid, kBatchThreads, 0, s>>>(L);
-        else batch_step_kernel<Q, true, STORE_F32><<<grid, kBatchThreads, 0, s>>>(L);
-    } else {
-        if (L.storage == STORE_F16) batch_step_kernel<Q, false, STORE_F16><<<grid, kBatchThreads, 0, s>>>(L);
-        else if (L.storage == STORE_BF16) batch_step_kernel<Q, false, STORE_BF16><<<grid, kBatchThreads, 0, s>>>(L);
-        else batch_step_kernel<Q, false, STORE_F32><<<grid, kBatchThreads, 0, s>>>(L);
-    }
+static cudaError_t launch_q(const BatchLaunch& L, dim3 grid, cudaStream_t s) {
+#define LBM_GROUP(S) \
+    launch_chained(L.general ? batch_step_kernel<Q, true, S> : batch_step_kernel<Q, false, S>, grid, dim3(kBatchThreads), 0, s, L)
+    if (L.storage == STORE_F16) return LBM_GROUP(STORE_F16);
+    if (L.storage == STORE_BF16) return LBM_GROUP(STORE_BF16);
+    return LBM_GROUP(STORE_F32);
+#undef LBM_GROUP
 }
 
 cudaError_t launch_batch_group(int Q, const BatchLaunch& L, cudaStream_t s) {
     if (L.n_cases <= 0) return cudaSuccess;
     const dim3 grid((unsigned)(L.ntx * L.nty), (unsigned)L.n_cases, (unsigned)L.ntz);
-    if (Q == 9) launch_q<9>(L, grid, s);
-    else launch_q<19>(L, grid, s);
-    return cudaGetLastError();
+    return Q == 9 ? launch_q<9>(L, grid, s) : launch_q<19>(L, grid, s);
 }
 
 __global__ void fill_plane0_kernel(float2* plane0, long long N) {

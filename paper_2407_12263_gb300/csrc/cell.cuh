@@ -18,6 +18,7 @@
 // (1/cs^2 = 3, 1/(2 cs^4) = 4.5).
 #pragma once
 
+#include "chain.cuh"
 #include "lattice.cuh"
 #include "lbm_internal.h"
 #include "storage.cuh"
@@ -442,6 +443,7 @@ __device__ __forceinline__ void step_cell(const Params& P, const void* __restric
     }
     macro_pressure<GEN>(P, m);
     collide<Q, GEN, S>(P, m, fb, gb);
+    chain_next();
 
     // streaming stores: the output is not re-read this step; one word per opposite pair
     __stcs(moment_plane(fg_out) + c, make_float2(fb[0], __int_as_float(phi_fx)));

@@ -39,6 +39,7 @@ template <int Q, int SCHEME, bool GEN, int S>
 __global__ void __launch_bounds__(kStepThreads, (step_min_blocks<S>()))
 step_kernel(const Params P, const void* __restrict__ fg_in, void* __restrict__ fg_out,
             const float* __restrict__ phi_fd) {
+    chain_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
@@ -50,6 +51,7 @@ step_kernel(const Params P, const void* __restrict__ fg_in, void* __restrict__ f
 template <int Q, int S, bool WALLS>
 __global__ void __launch_bounds__(kStepThreads, LBM_STEP_MINB)
 fd_phi_kernel(const Params P, const void* __restrict__ fg_in, float* __restrict__ phi) {
+    chain_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
@@ -59,6 +61,7 @@ fd_phi_kernel(const Params P, const void* __restrict__ fg_in, float* __restrict_
     float fb[Q], gb[Q];
     int phi_fx;
     pull<Q, false, S, WALLS>(P, fg_in, c, nb, fb, gb, phi_fx, WALLS ? make_wall_side(P, x, y, z) : WallSide{});
+    chain_next();
     phi[c] = gb[0];
 }
 
@@ -70,21 +73,25 @@ static dim3 step_grid(const Params& P) {
 }
 
 template <int Q, int S>
+static cudaError_t fd_phi_qs(const Params& P, const void* in, float* phi, cudaStream_t s) {
+    return launch_chained(P.walls ? fd_phi_kernel<Q, S, true> : fd_phi_kernel<Q, S, false>, step_grid(P), step_block(P), 0, s, P, in,
+                          phi);
+}
+
+template <int Q, int S>
 static cudaError_t step_qs(const Params& P, int scheme, const void* in, void* out, float* phi, cudaStream_t s,
                            int* launches) {
     const dim3 grid = step_grid(P), block = step_block(P);
     if (scheme == SCHEME_DF) {
-        if (P.general) step_kernel<Q, SCHEME_DF, true, S><<<grid, block, 0, s>>>(P, in, out, nullptr);
-        else step_kernel<Q, SCHEME_DF, false, S><<<grid, block, 0, s>>>(P, in, out, nullptr);
         *launches += 1;
-    } else {
-        if (P.walls) fd_phi_kernel<Q, S, true><<<grid, block, 0, s>>>(P, in, phi);
-        else fd_phi_kernel<Q, S, false><<<grid, block, 0, s>>>(P, in, phi);
-        if (P.general) step_kernel<Q, SCHEME_FD, true, S><<<grid, block, 0, s>>>(P, in, out, phi);
-        else step_kernel<Q, SCHEME_FD, false, S><<<grid, block, 0, s>>>(P, in, out, phi);
-        *launches += 2;
+        return launch_chained(P.general ? step_kernel<Q, SCHEME_DF, true, S> : step_kernel<Q, SCHEME_DF, false, S>, grid, block, 0, s,
+                              P, in, out, (const float*)nullptr);
     }
-    return cudaGetLastError();
+    *launches += 2;
+    const cudaError_t e = fd_phi_qs<Q, S>(P, in, phi, s);
+    if (e != cudaSuccess) return e;
+    return launch_chained(P.general ? step_kernel<Q, SCHEME_FD, true, S> : step_kernel<Q, SCHEME_FD, false, S>, grid, block, 0, s, P,
+                          in, out, (const float*)phi);
 }
 
 template <int Q>
@@ -101,23 +108,15 @@ cudaError_t launch_step(const Params& P, int scheme, const void* fg_in, void* fg
     return step_q<19>(P, scheme, fg_in, fg_out, phi_fd, s, launches);
 }
 
-template <int Q, int S>
-static void fd_phi_qs(const Params& P, const void* in, float* phi, cudaStream_t s) {
-    if (P.walls) fd_phi_kernel<Q, S, true><<<step_grid(P), step_block(P), 0, s>>>(P, in, phi);
-    else fd_phi_kernel<Q, S, false><<<step_grid(P), step_block(P), 0, s>>>(P, in, phi);
-}
-
 cudaError_t launch_fd_phi(const Params& P, const void* fg_in, float* phi_fd, cudaStream_t s) {
     if (P.Q == 9) {
-        if (P.storage == STORE_F16) fd_phi_qs<9, STORE_F16>(P, fg_in, phi_fd, s);
-        else if (P.storage == STORE_BF16) fd_phi_qs<9, STORE_BF16>(P, fg_in, phi_fd, s);
-        else fd_phi_qs<9, STORE_F32>(P, fg_in, phi_fd, s);
-    } else {
-        if (P.storage == STORE_F16) fd_phi_qs<19, STORE_F16>(P, fg_in, phi_fd, s);
-        else if (P.storage == STORE_BF16) fd_phi_qs<19, STORE_BF16>(P, fg_in, phi_fd, s);
-        else fd_phi_qs<19, STORE_F32>(P, fg_in, phi_fd, s);
+        if (P.storage == STORE_F16) return fd_phi_qs<9, STORE_F16>(P, fg_in, phi_fd, s);
+        if (P.storage == STORE_BF16) return fd_phi_qs<9, STORE_BF16>(P, fg_in, phi_fd, s);
+        return fd_phi_qs<9, STORE_F32>(P, fg_in, phi_fd, s);
     }
-    return cudaGetLastError();
+    if (P.storage == STORE_F16) return fd_phi_qs<19, STORE_F16>(P, fg_in, phi_fd, s);
+    if (P.storage == STORE_BF16) return fd_phi_qs<19, STORE_BF16>(P, fg_in, phi_fd, s);
+    return fd_phi_qs<19, STORE_F32>(P, fg_in, phi_fd, s);
 }
 
 }  // namespace lbm
