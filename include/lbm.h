@@ -10,7 +10,7 @@
  * FP32 storage), then one plane of words [nz][ny][nx] per opposite pair of populations (i, and
  * j with e_j = -e_i): per cell the pair of i then that of j, 16 B for FP32, 8 B for 16-bit.
  * Every step is one fused stream-collide kernel launch (difference-free scheme), or two
- * launches for the finite-difference variant.
+ * launches for the finite-difference variant; several steps of a small D2Q9 grid share one.
  *
  * Units are lattice units: dx = 1 and dt = 1 in every collision, moment and forcing
  * formula; the Courant number only enters the Lax-Wendroff propagation (Sec. 2.2).
@@ -227,7 +227,8 @@ int lbm_get_pops(lbm_ctx *ctx, double *f, double *g);
 int lbm_set_pops(lbm_ctx *ctx, const double *f, const double *g);
 
 /* Kernel launches issued by this handle since creation (one per step for the
- * difference-free scheme, two for the finite-difference variant, plus auxiliaries). */
+ * difference-free scheme, two for the finite-difference variant, plus auxiliaries; on small D2Q9
+ * grids, where a launch would take longer than its step, one for several steps). */
 long long lbm_launch_count(const lbm_ctx *ctx);
 
 /* tau_phi the handle resolved from (tau_g, M). */
