@@ -266,12 +266,18 @@ __device__ __forceinline__ void macro_interface_df(const Params& P, Macro& m) {
     m.gphi[2] = P.grad_s * m.S[2] - P.grad_k * kz;
 }
 
+// |v|^2 of the finite-difference variant, with the order of its roundings written out: every kernel that
+// compiles that variant gives the same bits.
+__device__ __forceinline__ float norm2_fd(float x, float y, float z) {
+    return __fmaf_rn(z, z, __fmaf_rn(x, x, __fmul_rn(y, y)));
+}
+
 // Finite-difference variant (Sec. 3.4): n = grad phi / |grad phi| with grad phi given.
 __device__ __forceinline__ void macro_interface_fd(const Params& P, float gx, float gy, float gz, Macro& m) {
     m.gphi[0] = gx;
     m.gphi[1] = gy;
     m.gphi[2] = gz;
-    const float g2 = gx * gx + gy * gy + gz * gz;
+    const float g2 = norm2_fd(gx, gy, gz);
     const float r = (g2 > kNormalGuard) ? rsqrtf(g2) : 0.f;
     m.n[0] = gx * r;
     m.n[1] = gy * r;
@@ -283,31 +289,32 @@ __device__ __forceinline__ void macro_interface_fd(const Params& P, float gx, fl
 }
 
 // Pressure (Eq. pressure): p/cs^2 = sum fbar_i + u . grad rho / 2, held as P = p/cs^2 - w0.
-template <bool GEN>
+template <bool GEN, int SCHEME = SCHEME_DF>
 __device__ __forceinline__ void macro_pressure(const Params& P, Macro& m) {
     m.P = m.Pbar;
     if (GEN) m.P += 0.5f * P.drho * (m.u[0] * m.gphi[0] + m.u[1] * m.gphi[1] + m.u[2] * m.gphi[2]);
-    m.gnorm = sqrtf(m.gphi[0] * m.gphi[0] + m.gphi[1] * m.gphi[1] + m.gphi[2] * m.gphi[2]);
+    if (SCHEME == SCHEME_FD) m.gnorm = sqrtf(norm2_fd(m.gphi[0], m.gphi[1], m.gphi[2]));
+    else m.gnorm = sqrtf(m.gphi[0] * m.gphi[0] + m.gphi[1] * m.gphi[1] + m.gphi[2] * m.gphi[2]);
 }
 
 // Isotropic central difference of the propagated phi field (Sec. 3.4):
 // grad phi = sum_{i != 0} t_i e_i [phi(x + e_i) - phi(x - e_i)] / (2 cs^2)
 //          = 3 sum_{i != 0} t_i e_i phi(x + e_i)   (the velocity set is symmetric).
-// The plane holds phi - phi_ref; the constant drops out of the difference.
+// The plane holds phi - phi_ref; the constant drops out of the difference. fd_term: one term of it.
+template <int Q>
+__device__ __forceinline__ void fd_term(int i, float v, float& gx, float& gy, float& gz) {
+    const float w = Lat<Q>::w(i);
+    if (Lat<Q>::cx(i) != 0) gx = __fmaf_rn(Lat<Q>::cx(i) > 0 ? w : -w, v, gx);
+    if (Lat<Q>::cy(i) != 0) gy = __fmaf_rn(Lat<Q>::cy(i) > 0 ? w : -w, v, gy);
+    if (Lat<Q>::cz(i) != 0) gz = __fmaf_rn(Lat<Q>::cz(i) > 0 ? w : -w, v, gz);
+}
+
 template <int Q>
 __device__ __forceinline__ void fd_gradient(const float* __restrict__ phi, int c, const Nbr& nb,
                                             float& gx, float& gy, float& gz) {
     gx = gy = gz = 0.f;
 #pragma unroll
-    for (int i = 1; i < Q; ++i) {
-        const float v = Lat<Q>::w(i) * __ldg(phi + c + link_offset<Q>(nb, i, +1));
-        if (Lat<Q>::cx(i) > 0) gx += v;
-        if (Lat<Q>::cx(i) < 0) gx -= v;
-        if (Lat<Q>::cy(i) > 0) gy += v;
-        if (Lat<Q>::cy(i) < 0) gy -= v;
-        if (Lat<Q>::cz(i) > 0) gz += v;
-        if (Lat<Q>::cz(i) < 0) gz -= v;
-    }
+    for (int i = 1; i < Q; ++i) fd_term<Q>(i, __ldg(phi + c + link_offset<Q>(nb, i, +1)), gx, gy, gz);
     gx *= 3.f;
     gy *= 3.f;
     gz *= 3.f;
@@ -441,7 +448,7 @@ __device__ __forceinline__ void step_cell(const Params& P, const void* __restric
         fd_gradient<Q>(phi_fd, c, GEN ? mirror_at_walls(nb, ws) : nb, gx, gy, gz);
         macro_interface_fd(P, gx, gy, gz, m);
     }
-    macro_pressure<GEN>(P, m);
+    macro_pressure<GEN, SCHEME>(P, m);
     collide<Q, GEN, S>(P, m, fb, gb);
     chain_next();
 

@@ -20,9 +20,7 @@
 
 namespace lbm {
 
-// Thread block: 128 threads, one cell per thread, x fastest. The host picks the shape: one
-// 128-cell row per block where rows are at least that long, else 32 x 4 (a warp spans 32
-// consecutive cells of a row either way). With FP32 storage the register budget allows 4
+// Thread block: 128 threads, one cell per thread, x fastest (step_shape has the shapes). With FP32 storage the register budget allows 4
 // blocks (16 warps) per SM: the difference-free step needs ~122 registers and runs at that
 // occupancy with every (f, g) load of a cell in flight. A 16-bit cell moves half the bytes, so
 // the same bandwidth needs more cells in flight: the 16-bit steps are held to 96 registers for
@@ -35,27 +33,46 @@ constexpr int step_min_blocks() {
     return S == STORE_F32 ? LBM_STEP_MINB : 5;
 }
 
-template <int Q, int SCHEME, bool GEN, int S>
+// i / nx (nx > 1) for i < 2^31 as a product: mul = ceil(2^(32 + shift) / nx), 2^shift < nx <= 2^(shift + 1). The
+// excess mul nx - 2^(32 + shift) is below nx <= 2^(shift + 1), so i times it stays below 2^(32 + shift).
+struct RowDiv {
+    unsigned mul;
+    int shift;
+};
+
+// The cell of a thread, false beyond the grid. PACKED: blocks of 128 cells that follow one another in
+// a plane, whatever its rows, instead of blocks of whole rows or of 32 x 4 cells.
+template <bool PACKED>
+__device__ __forceinline__ bool own_cell(const Params& P, const RowDiv& d, int& x, int& y, int& z) {
+    z = blockIdx.z;
+    if (PACKED) {
+        const unsigned i = blockIdx.x * kStepThreads + threadIdx.x;
+        y = (int)(__umulhi(i, d.mul) >> d.shift);
+        x = (int)i - y * P.nx;
+        return y < P.ny;
+    }
+    x = blockIdx.x * blockDim.x + threadIdx.x;
+    y = blockIdx.y * blockDim.y + threadIdx.y;
+    return x < P.nx && y < P.ny;
+}
+
+template <int Q, int SCHEME, bool GEN, int S, bool PACKED>
 __global__ void __launch_bounds__(kStepThreads, (step_min_blocks<S>()))
 step_kernel(const Params P, const void* __restrict__ fg_in, void* __restrict__ fg_out,
-            const float* __restrict__ phi_fd) {
+            const float* __restrict__ phi_fd, const RowDiv d) {
     chain_begin();
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    if (x >= P.nx || y >= P.ny) return;
+    int x, y, z;
+    if (!own_cell<PACKED>(P, d, x, y, z)) return;
     step_cell<Q, SCHEME, GEN, S>(P, fg_in, fg_out, phi_fd, x, y, z);
 }
 
 // Finite-difference variant, pass 1: the propagated phi (held as phi - phi_ref), one FP32 plane.
-template <int Q, int S, bool WALLS>
+template <int Q, int S, bool WALLS, bool PACKED>
 __global__ void __launch_bounds__(kStepThreads, LBM_STEP_MINB)
-fd_phi_kernel(const Params P, const void* __restrict__ fg_in, float* __restrict__ phi) {
+fd_phi_kernel(const Params P, const void* __restrict__ fg_in, float* __restrict__ phi, const RowDiv d) {
     chain_begin();
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    if (x >= P.nx || y >= P.ny) return;
+    int x, y, z;
+    if (!own_cell<PACKED>(P, d, x, y, z)) return;
     const Nbr nb = make_nbr(P, x, y, z);
     const int c = (z * P.ny + y) * P.nx + x;
     float fb[Q], gb[Q];
@@ -65,41 +82,72 @@ fd_phi_kernel(const Params P, const void* __restrict__ fg_in, float* __restrict_
     phi[c] = gb[0];
 }
 
-static dim3 step_block(const Params& P) { return P.nx >= 128 ? dim3(128, 1, 1) : dim3(32, 4, 1); }
+// Blocks of one 128-cell row where rows are at least that long, else 32 x 4 (a warp spans 32 consecutive
+// cells of a row either way); where such blocks would stand over the grid's edges, packed ones, which
+// leave no lane idle but in a plane's last block. Packed blocks cost a product per cell to find the
+// row: 0.4% at 128^3 (59.98 against 60.36 us FP16, 93.16 against 93.39 FP32), so whole blocks stay where
+// they fit. Where they do not, packed ones were faster at every size tried (us per step):
+//   grid              33^3  33^3   97x96x96  126^3  130^3  130^3   200^3   200^3   94x75x301  600^2  330x270
+//                     FP16  FP32*  FP32*     FP16   FP16   FP32    BF16    FP32    BF16*      FP32   FP32
+//   whole blocks      3.31  4.30   51.2      61.1   84.6   115.5   266.0   373.6   74.1       6.13   2.87
+//   packed            2.42  3.30   44.0      60.0   65.7   99.7    231.2   349.1   72.6       5.85   2.65
+// (* walls and a density ratio)
+struct StepShape {
+    dim3 block, grid;
+    bool packed;
+    RowDiv d;
+};
 
-static dim3 step_grid(const Params& P) {
-    const dim3 b = step_block(P);
-    return dim3((P.nx + b.x - 1) / b.x, (P.ny + b.y - 1) / b.y, P.nz);
+static StepShape step_shape(const Params& P) {
+    StepShape h;
+    h.block = P.nx >= 128 ? dim3(128, 1, 1) : dim3(32, 4, 1);
+    h.grid = dim3((P.nx + h.block.x - 1) / h.block.x, (P.ny + h.block.y - 1) / h.block.y, P.nz);
+    const unsigned blocks = (unsigned)((P.nxy + kStepThreads - 1) / kStepThreads);
+    h.packed = P.nx > 1 && blocks < h.grid.x * h.grid.y;
+    h.d = RowDiv{0u, 0};
+    if (h.packed) {
+        h.block = dim3(kStepThreads, 1, 1);
+        h.grid = dim3(blocks, 1, P.nz);
+        while ((2 << h.d.shift) < P.nx) ++h.d.shift;
+        h.d.mul = (unsigned)(((1ull << (32 + h.d.shift)) + P.nx - 1) / P.nx);
+    }
+    return h;
 }
 
-template <int Q, int S>
-static cudaError_t fd_phi_qs(const Params& P, const void* in, float* phi, cudaStream_t s) {
-    return launch_chained(P.walls ? fd_phi_kernel<Q, S, true> : fd_phi_kernel<Q, S, false>, step_grid(P), step_block(P), 0, s, P, in,
-                          phi);
+template <int Q, int S, bool PACKED>
+static cudaError_t fd_phi_qs(const Params& P, const StepShape& h, const void* in, float* phi, cudaStream_t s) {
+    return launch_chained(P.walls ? fd_phi_kernel<Q, S, true, PACKED> : fd_phi_kernel<Q, S, false, PACKED>, h.grid, h.block, 0, s, P, in,
+                          phi, h.d);
 }
 
-template <int Q, int S>
-static cudaError_t step_qs(const Params& P, int scheme, const void* in, void* out, float* phi, cudaStream_t s,
+template <int Q, int S, bool PACKED>
+static cudaError_t step_qs(const Params& P, const StepShape& h, int scheme, const void* in, void* out, float* phi, cudaStream_t s,
                            int* launches) {
-    const dim3 grid = step_grid(P), block = step_block(P);
     if (scheme == SCHEME_DF) {
         *launches += 1;
-        return launch_chained(P.general ? step_kernel<Q, SCHEME_DF, true, S> : step_kernel<Q, SCHEME_DF, false, S>, grid, block, 0, s,
-                              P, in, out, (const float*)nullptr);
+        return launch_chained(P.general ? step_kernel<Q, SCHEME_DF, true, S, PACKED> : step_kernel<Q, SCHEME_DF, false, S, PACKED>,
+                              h.grid, h.block, 0, s, P, in, out, (const float*)nullptr, h.d);
     }
     *launches += 2;
-    const cudaError_t e = fd_phi_qs<Q, S>(P, in, phi, s);
+    const cudaError_t e = fd_phi_qs<Q, S, PACKED>(P, h, in, phi, s);
     if (e != cudaSuccess) return e;
-    return launch_chained(P.general ? step_kernel<Q, SCHEME_FD, true, S> : step_kernel<Q, SCHEME_FD, false, S>, grid, block, 0, s, P,
-                          in, out, (const float*)phi);
+    return launch_chained(P.general ? step_kernel<Q, SCHEME_FD, true, S, PACKED> : step_kernel<Q, SCHEME_FD, false, S, PACKED>, h.grid,
+                          h.block, 0, s, P, in, out, (const float*)phi, h.d);
+}
+
+template <int Q, int S>
+static cudaError_t step_s(const Params& P, int scheme, const void* in, void* out, float* phi, cudaStream_t s, int* launches) {
+    const StepShape h = step_shape(P);
+    return h.packed ? step_qs<Q, S, true>(P, h, scheme, in, out, phi, s, launches)
+                    : step_qs<Q, S, false>(P, h, scheme, in, out, phi, s, launches);
 }
 
 template <int Q>
 static cudaError_t step_q(const Params& P, int scheme, const void* in, void* out, float* phi, cudaStream_t s,
                           int* launches) {
-    if (P.storage == STORE_F16) return step_qs<Q, STORE_F16>(P, scheme, in, out, phi, s, launches);
-    if (P.storage == STORE_BF16) return step_qs<Q, STORE_BF16>(P, scheme, in, out, phi, s, launches);
-    return step_qs<Q, STORE_F32>(P, scheme, in, out, phi, s, launches);
+    if (P.storage == STORE_F16) return step_s<Q, STORE_F16>(P, scheme, in, out, phi, s, launches);
+    if (P.storage == STORE_BF16) return step_s<Q, STORE_BF16>(P, scheme, in, out, phi, s, launches);
+    return step_s<Q, STORE_F32>(P, scheme, in, out, phi, s, launches);
 }
 
 cudaError_t launch_step(const Params& P, int scheme, const void* fg_in, void* fg_out, float* phi_fd, cudaStream_t s,
@@ -108,15 +156,21 @@ cudaError_t launch_step(const Params& P, int scheme, const void* fg_in, void* fg
     return step_q<19>(P, scheme, fg_in, fg_out, phi_fd, s, launches);
 }
 
+template <int Q, int S>
+static cudaError_t fd_phi_s(const Params& P, const void* in, float* phi, cudaStream_t s) {
+    const StepShape h = step_shape(P);
+    return h.packed ? fd_phi_qs<Q, S, true>(P, h, in, phi, s) : fd_phi_qs<Q, S, false>(P, h, in, phi, s);
+}
+
+template <int Q>
+static cudaError_t fd_phi_q(const Params& P, const void* in, float* phi, cudaStream_t s) {
+    if (P.storage == STORE_F16) return fd_phi_s<Q, STORE_F16>(P, in, phi, s);
+    if (P.storage == STORE_BF16) return fd_phi_s<Q, STORE_BF16>(P, in, phi, s);
+    return fd_phi_s<Q, STORE_F32>(P, in, phi, s);
+}
+
 cudaError_t launch_fd_phi(const Params& P, const void* fg_in, float* phi_fd, cudaStream_t s) {
-    if (P.Q == 9) {
-        if (P.storage == STORE_F16) return fd_phi_qs<9, STORE_F16>(P, fg_in, phi_fd, s);
-        if (P.storage == STORE_BF16) return fd_phi_qs<9, STORE_BF16>(P, fg_in, phi_fd, s);
-        return fd_phi_qs<9, STORE_F32>(P, fg_in, phi_fd, s);
-    }
-    if (P.storage == STORE_F16) return fd_phi_qs<19, STORE_F16>(P, fg_in, phi_fd, s);
-    if (P.storage == STORE_BF16) return fd_phi_qs<19, STORE_BF16>(P, fg_in, phi_fd, s);
-    return fd_phi_qs<19, STORE_F32>(P, fg_in, phi_fd, s);
+    return P.Q == 9 ? fd_phi_q<9>(P, fg_in, phi_fd, s) : fd_phi_q<19>(P, fg_in, phi_fd, s);
 }
 
 }  // namespace lbm

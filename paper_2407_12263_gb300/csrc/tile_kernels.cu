@@ -68,15 +68,7 @@ __device__ __forceinline__ void tile_pull(const Params& P, const typename Store<
 __device__ __forceinline__ void tile_gradient(const float* phi, int c, const Nbr& nb, float& gx, float& gy, float& gz) {
     gx = gy = gz = 0.f;
 #pragma unroll
-    for (int i = 1; i < Q9; ++i) {
-        const float v = Lat<Q9>::w(i) * phi[c + link_offset<Q9>(nb, i, +1)];
-        if (Lat<Q9>::cx(i) > 0) gx += v;
-        if (Lat<Q9>::cx(i) < 0) gx -= v;
-        if (Lat<Q9>::cy(i) > 0) gy += v;
-        if (Lat<Q9>::cy(i) < 0) gy -= v;
-        if (Lat<Q9>::cz(i) > 0) gz += v;
-        if (Lat<Q9>::cz(i) < 0) gz -= v;
-    }
+    for (int i = 1; i < Q9; ++i) fd_term<Q9>(i, phi[c + link_offset<Q9>(nb, i, +1)], gx, gy, gz);
     gx *= 3.f;
     gy *= 3.f;
     gz *= 3.f;
@@ -138,7 +130,7 @@ tile_step_kernel(const Params P, const void* __restrict__ fg_in, void* __restric
                 tile_gradient(phi, c, GEN ? mirror_at_walls(nb, ws) : nb, dx, dy, dz);
                 macro_interface_fd(P, dx, dy, dz, m);
             }
-            macro_pressure<GEN>(P, m);
+            macro_pressure<GEN, SCHEME>(P, m);
             collide<Q9, GEN, S>(P, m, fb, gb);
         }
         if (t < steps) {
