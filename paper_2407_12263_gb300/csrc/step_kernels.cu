@@ -40,12 +40,12 @@ struct RowDiv {
     int shift;
 };
 
-// The cell of a thread, false beyond the grid. PACKED: blocks of 128 cells that follow one another in
+// The cell of a thread, false beyond the grid. PACK: blocks of 128 cells that follow one another in
 // a plane, whatever its rows, instead of blocks of whole rows or of 32 x 4 cells.
-template <bool PACKED>
+template <bool PACK>
 __device__ __forceinline__ bool own_cell(const Params& P, const RowDiv& d, int& x, int& y, int& z) {
     z = blockIdx.z;
-    if (PACKED) {
+    if (PACK) {
         const unsigned i = blockIdx.x * kStepThreads + threadIdx.x;
         y = (int)(__umulhi(i, d.mul) >> d.shift);
         x = (int)i - y * P.nx;
@@ -56,28 +56,34 @@ __device__ __forceinline__ bool own_cell(const Params& P, const RowDiv& d, int& 
     return x < P.nx && y < P.ny;
 }
 
-template <int Q, int SCHEME, bool GEN, int S, bool PACKED>
+// How a step's blocks lie and address: whole rows or 32 x 4 cells, packed, or whole blocks with 64-bit
+// addresses for the 16-bit D3Q19 planes of 4 GiB and more (2^29 cells), where a byte offset does not fit.
+enum StepForm { WHOLE = 0, PACKED = 1, WIDE = 2 };
+template <int Q, int S>
+constexpr bool narrow_form(int form) { return Q == 19 && S != STORE_F32 && form != WIDE; }
+
+template <int Q, int SCHEME, bool GEN, int S, int FORM>
 __global__ void __launch_bounds__(kStepThreads, (step_min_blocks<S>()))
 step_kernel(const Params P, const void* __restrict__ fg_in, void* __restrict__ fg_out,
             const float* __restrict__ phi_fd, const RowDiv d) {
     chain_begin();
     int x, y, z;
-    if (!own_cell<PACKED>(P, d, x, y, z)) return;
-    step_cell<Q, SCHEME, GEN, S>(P, fg_in, fg_out, phi_fd, x, y, z);
+    if (!own_cell<FORM == PACKED>(P, d, x, y, z)) return;
+    step_cell<Q, SCHEME, GEN, S, narrow_form<Q, S>(FORM)>(P, fg_in, fg_out, phi_fd, x, y, z);
 }
 
 // Finite-difference variant, pass 1: the propagated phi (held as phi - phi_ref), one FP32 plane.
-template <int Q, int S, bool WALLS, bool PACKED>
+template <int Q, int S, bool WALLS, int FORM>
 __global__ void __launch_bounds__(kStepThreads, LBM_STEP_MINB)
 fd_phi_kernel(const Params P, const void* __restrict__ fg_in, float* __restrict__ phi, const RowDiv d) {
     chain_begin();
     int x, y, z;
-    if (!own_cell<PACKED>(P, d, x, y, z)) return;
+    if (!own_cell<FORM == PACKED>(P, d, x, y, z)) return;
     const Nbr nb = make_nbr(P, x, y, z);
     const int c = (z * P.ny + y) * P.nx + x;
     float fb[Q], gb[Q];
     int phi_fx;
-    pull<Q, false, S, WALLS>(P, fg_in, c, nb, fb, gb, phi_fx, WALLS ? make_wall_side(P, x, y, z) : WallSide{});
+    pull<Q, false, S, WALLS, false, narrow_form<Q, S>(FORM)>(P, fg_in, c, nb, fb, gb, phi_fx, WALLS ? make_wall_side(P, x, y, z) : WallSide{});
     chain_next();
     phi[c] = gb[0];
 }
@@ -94,7 +100,7 @@ fd_phi_kernel(const Params P, const void* __restrict__ fg_in, float* __restrict_
 // (* walls and a density ratio)
 struct StepShape {
     dim3 block, grid;
-    bool packed;
+    StepForm form;
     RowDiv d;
 };
 
@@ -103,9 +109,10 @@ static StepShape step_shape(const Params& P) {
     h.block = P.nx >= 128 ? dim3(128, 1, 1) : dim3(32, 4, 1);
     h.grid = dim3((P.nx + h.block.x - 1) / h.block.x, (P.ny + h.block.y - 1) / h.block.y, P.nz);
     const unsigned blocks = (unsigned)((P.nxy + kStepThreads - 1) / kStepThreads);
-    h.packed = P.nx > 1 && blocks < h.grid.x * h.grid.y;
+    h.form = P.nx > 1 && blocks < h.grid.x * h.grid.y ? PACKED : WHOLE;
+    if (P.Q == 19 && P.storage != STORE_F32 && P.N >= (1ll << 29)) h.form = WIDE;
     h.d = RowDiv{0u, 0};
-    if (h.packed) {
+    if (h.form == PACKED) {
         h.block = dim3(kStepThreads, 1, 1);
         h.grid = dim3(blocks, 1, P.nz);
         while ((2 << h.d.shift) < P.nx) ++h.d.shift;
@@ -114,32 +121,34 @@ static StepShape step_shape(const Params& P) {
     return h;
 }
 
-template <int Q, int S, bool PACKED>
+template <int Q, int S, int FORM>
 static cudaError_t fd_phi_qs(const Params& P, const StepShape& h, const void* in, float* phi, cudaStream_t s) {
-    return launch_chained(P.walls ? fd_phi_kernel<Q, S, true, PACKED> : fd_phi_kernel<Q, S, false, PACKED>, h.grid, h.block, 0, s, P, in,
+    return launch_chained(P.walls ? fd_phi_kernel<Q, S, true, FORM> : fd_phi_kernel<Q, S, false, FORM>, h.grid, h.block, 0, s, P, in,
                           phi, h.d);
 }
 
-template <int Q, int S, bool PACKED>
+template <int Q, int S, int FORM>
 static cudaError_t step_qs(const Params& P, const StepShape& h, int scheme, const void* in, void* out, float* phi, cudaStream_t s,
                            int* launches) {
     if (scheme == SCHEME_DF) {
         *launches += 1;
-        return launch_chained(P.general ? step_kernel<Q, SCHEME_DF, true, S, PACKED> : step_kernel<Q, SCHEME_DF, false, S, PACKED>,
+        return launch_chained(P.general ? step_kernel<Q, SCHEME_DF, true, S, FORM> : step_kernel<Q, SCHEME_DF, false, S, FORM>,
                               h.grid, h.block, 0, s, P, in, out, (const float*)nullptr, h.d);
     }
     *launches += 2;
-    const cudaError_t e = fd_phi_qs<Q, S, PACKED>(P, h, in, phi, s);
+    const cudaError_t e = fd_phi_qs<Q, S, FORM>(P, h, in, phi, s);
     if (e != cudaSuccess) return e;
-    return launch_chained(P.general ? step_kernel<Q, SCHEME_FD, true, S, PACKED> : step_kernel<Q, SCHEME_FD, false, S, PACKED>, h.grid,
+    return launch_chained(P.general ? step_kernel<Q, SCHEME_FD, true, S, FORM> : step_kernel<Q, SCHEME_FD, false, S, FORM>, h.grid,
                           h.block, 0, s, P, in, out, (const float*)phi, h.d);
 }
 
 template <int Q, int S>
 static cudaError_t step_s(const Params& P, int scheme, const void* in, void* out, float* phi, cudaStream_t s, int* launches) {
     const StepShape h = step_shape(P);
-    return h.packed ? step_qs<Q, S, true>(P, h, scheme, in, out, phi, s, launches)
-                    : step_qs<Q, S, false>(P, h, scheme, in, out, phi, s, launches);
+    if constexpr (narrow_form<Q, S>(WHOLE))
+        if (h.form == WIDE) return step_qs<Q, S, WIDE>(P, h, scheme, in, out, phi, s, launches);
+    return h.form == PACKED ? step_qs<Q, S, PACKED>(P, h, scheme, in, out, phi, s, launches)
+                            : step_qs<Q, S, WHOLE>(P, h, scheme, in, out, phi, s, launches);
 }
 
 template <int Q>
@@ -159,7 +168,9 @@ cudaError_t launch_step(const Params& P, int scheme, const void* fg_in, void* fg
 template <int Q, int S>
 static cudaError_t fd_phi_s(const Params& P, const void* in, float* phi, cudaStream_t s) {
     const StepShape h = step_shape(P);
-    return h.packed ? fd_phi_qs<Q, S, true>(P, h, in, phi, s) : fd_phi_qs<Q, S, false>(P, h, in, phi, s);
+    if constexpr (narrow_form<Q, S>(WHOLE))
+        if (h.form == WIDE) return fd_phi_qs<Q, S, WIDE>(P, h, in, phi, s);
+    return h.form == PACKED ? fd_phi_qs<Q, S, PACKED>(P, h, in, phi, s) : fd_phi_qs<Q, S, WHOLE>(P, h, in, phi, s);
 }
 
 template <int Q>
