@@ -102,7 +102,7 @@ int lbm_restart_from_coarse(lbm_ctx *ctx, int factor, const float *coarse, doubl
  * u: device FP32 [3][nz][ny][nx] (components x, y, z, x fastest), replaced in place; grid
  * (nx, ny, nz), each extent 1 .. 512; work: device scratch of at least
  * lbm_project_workspace_bytes(grid) bytes (caller-owned; nothing is allocated), 16-byte
- * aligned; stream: cudaStream_t or NULL (the legacy default stream). Asynchronous: 9
+ * aligned; stream: cudaStream_t or NULL (the legacy default stream). Asynchronous: 8
  * kernel launches on the stream. Returns LBM_EINVAL for a NULL pointer, an extent outside
  * 1 .. 512, a misaligned pointer or too small a workspace (nothing is launched), LBM_ECUDA if a
  * launch fails. */

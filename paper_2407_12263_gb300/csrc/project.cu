@@ -15,7 +15,13 @@
 // FP32, in a fixed order (the same bits on every run). Lines along x are rows; along y and z a
 // block takes 8 neighbouring x positions, so every global access covers 8 consecutive values.
 // The coarse grids this serves are small (64^3 for a 256^3 lattice at factor 4): the direct sums
-// cost n complex multiply-adds per output, 6 passes of 3 components.
+// cost n complex multiply-adds per output, 6 passes of 3 components. At 64^3 a pass takes 20 us, a third
+// of it multiply-adds, the rest their loads from shared memory and the twiddles' index; below 32^3 the
+// launches are what it takes, so the kernels follow one another without gaps (chain.cuh). The whole
+// projection at 64^3 went from 154 to 132 us with that, with eight terms unrolled and without the sums that
+// a real input or output does not need, at 40^3 from 56 to 39, at 16^3 from 33 to 17; an odd length of
+// lines in shared memory took 5 x 511 x 3 from 765 to 288. Several lines or outputs per thread gained at
+// 128^3 only (1644 -> 1340 us) and lost up to a half on thin grids, whose lines then fill fewer warps.
 #include <cuda_runtime.h>
 
 #include <climits>
@@ -23,6 +29,7 @@
 
 #include "../../include/lbm.h"
 #include "../../include/lbm_surrogate.h"
+#include "chain.cuh"
 #include "surrogate.h"
 
 namespace lbm {
@@ -30,7 +37,7 @@ namespace proj {
 
 constexpr int kLines = 8;       // lines per block
 constexpr int kThreads = 256;
-constexpr int kMaxExtent = 512;  // (kLines + 1) (n + 1) float2 of shared memory stay below 48 KB
+constexpr int kMaxExtent = 512;  // (kLines + 1) (n | 1) float2 of shared memory stay below 48 KB
 
 __host__ __device__ inline size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 
@@ -44,6 +51,8 @@ inline size_t workspace_bytes(int nx, int ny, int nz) {
 // w[m] = exp(-2 pi i m / n) for each axis, from the FP64 cospi / sinpi, which are exactly 0 and
 // +-1 where 2 m / n is an integer or a half-integer.
 __global__ void twiddle_kernel(float2* tw, int nx, int ny, int nz) {
+    chain_begin();
+    chain_next();
     const int total = nx + ny + nz;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
         const int n = t < nx ? nx : t < nx + ny ? ny : nz;
@@ -55,15 +64,16 @@ __global__ void twiddle_kernel(float2* tw, int nx, int ny, int nz) {
 }
 
 // One transform pass along AXIS (0 x, 1 y, 2 z) over the spectrum W (in place). inverse: the
-// conjugate twiddles. in_real (pass along x only): read the real field [3][N] instead of W.
-// out_real (pass along x only): write scale times the real part to [3][N] instead of W.
-template <int AXIS>
+// conjugate twiddles. REAL_IN (pass along x only): read the real field [3][N] instead of W, whose
+// zero imaginary parts add nothing to the sums and are left out. REAL_OUT (pass along x only): write
+// scale times the real part to [3][N] instead of W, and sum nothing else.
+template <int AXIS, bool REAL_IN, bool REAL_OUT>
 __global__ void __launch_bounds__(kThreads) dft_kernel(float2* __restrict__ W, const float2* __restrict__ tw_axis,
                                                        const float* __restrict__ in_real, float* __restrict__ out_real,
                                                        int nx, int ny, int nz, int inverse, float scale) {
     extern __shared__ float2 sm[];
     const int n = AXIS == 0 ? nx : AXIS == 1 ? ny : nz;
-    const int ld = n + 1;  // padded line: the 8 lines of a warp's reads sit in different banks
+    const int ld = n | 1;  // odd: the 8 lines of a warp's reads sit in different banks
     float2* tw = sm;
     float2* tile = sm + ld;
     long long base, lstride, estride;
@@ -89,6 +99,7 @@ __global__ void __launch_bounds__(kThreads) dft_kernel(float2* __restrict__ W, c
         }
         lstride = 1;
     }
+    chain_begin();
     for (int m = threadIdx.x; m < n; m += blockDim.x) {
         const float2 w = tw_axis[m];
         tw[m] = inverse ? make_float2(w.x, -w.y) : w;
@@ -99,32 +110,36 @@ __global__ void __launch_bounds__(kThreads) dft_kernel(float2* __restrict__ W, c
         float2 v = make_float2(0.f, 0.f);
         if (l < nl) {
             const long long o = base + l * lstride + j * estride;
-            v = in_real ? make_float2(in_real[o], 0.f) : W[o];
+            v = REAL_IN ? make_float2(in_real[o], 0.f) : W[o];
         }
         tile[l * ld + j] = v;
     }
     __syncthreads();
+    chain_next();
     for (int t = threadIdx.x; t < kLines * n; t += blockDim.x) {
         const int l = t % kLines, k = t / kLines;
         if (l >= nl) continue;
         const float2* x = tile + l * ld;
         float re = 0.f, im = 0.f;
         int m = 0;  // j k mod n
+#pragma unroll 8
         for (int j = 0; j < n; ++j) {
             const float2 a = x[j], w = tw[m];
-            re = fmaf(a.x, w.x, fmaf(-a.y, w.y, re));
-            im = fmaf(a.x, w.y, fmaf(a.y, w.x, im));
+            re = fmaf(a.x, w.x, REAL_IN ? re : fmaf(-a.y, w.y, re));
+            if (!REAL_OUT) im = fmaf(a.x, w.y, REAL_IN ? im : fmaf(a.y, w.x, im));
             m += k;
             if (m >= n) m -= n;
         }
         const long long o = base + l * lstride + k * estride;
-        if (out_real) out_real[o] = re * scale;
+        if (REAL_OUT) out_real[o] = re * scale;
         else W[o] = make_float2(re, im);
     }
 }
 
 // U <- U - s (s . U) / |s|^2 for every mode (kx, ky, kz); s_a = sin(2 pi k_a / n_a) = -Im w_a[k_a].
 __global__ void project_modes_kernel(float2* __restrict__ W, const float2* __restrict__ tw, int nx, int ny, int nz) {
+    chain_begin();
+    chain_next();
     const long long N = (long long)nx * ny * nz;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
         const int kx = (int)(i % nx), ky = (int)((i / nx) % ny), kz = (int)(i / ((long long)nx * ny));
@@ -140,40 +155,40 @@ __global__ void project_modes_kernel(float2* __restrict__ W, const float2* __res
     }
 }
 
-inline size_t dft_smem(int n) { return (size_t)(kLines + 1) * (n + 1) * sizeof(float2); }
+inline size_t dft_smem(int n) { return (size_t)(kLines + 1) * (n | 1) * sizeof(float2); }
 
-template <int AXIS>
+template <int AXIS, bool REAL_IN, bool REAL_OUT>
 cudaError_t dft(float2* W, const float2* tw, const float* in_real, float* out_real, int nx, int ny, int nz, int inverse,
                 float scale, cudaStream_t s) {
     const int n = AXIS == 0 ? nx : AXIS == 1 ? ny : nz;
     const long long blocks = AXIS == 0 ? (3ll * nz * ny + kLines - 1) / kLines
                                        : 3ll * (AXIS == 1 ? nz : ny) * ((nx + kLines - 1) / kLines);
     const float2* tw_axis = tw + (AXIS == 0 ? 0 : AXIS == 1 ? nx : nx + ny);
-    dft_kernel<AXIS><<<(unsigned)blocks, kThreads, dft_smem(n), s>>>(W, tw_axis, in_real, out_real, nx, ny, nz, inverse,
-                                                                     scale);
-    return cudaGetLastError();
+    return launch_chained(dft_kernel<AXIS, REAL_IN, REAL_OUT>, dim3((unsigned)blocks), dim3(kThreads), dft_smem(n), s, W, tw_axis,
+                          in_real, out_real, nx, ny, nz, inverse, scale);
 }
 
 }  // namespace proj
 
-// The whole projection of u [3][nz][ny][nx] in place: 9 launches on stream s.
+// The whole projection of u [3][nz][ny][nx] in place: 8 launches on stream s.
 cudaError_t launch_project_solenoidal(float* u, int nx, int ny, int nz, void* work, cudaStream_t s) {
     using namespace proj;
     float2* tw = static_cast<float2*>(work);
     float2* W = reinterpret_cast<float2*>(static_cast<char*>(work) + twiddle_bytes(nx, ny, nz));
     const long long N = (long long)nx * ny * nz;
     cudaError_t e;
-    twiddle_kernel<<<1, kThreads, 0, s>>>(tw, nx, ny, nz);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = dft<0>(W, tw, u, nullptr, nx, ny, nz, 0, 1.f, s)) != cudaSuccess) return e;
-    if ((e = dft<1>(W, tw, nullptr, nullptr, nx, ny, nz, 0, 1.f, s)) != cudaSuccess) return e;
-    if ((e = dft<2>(W, tw, nullptr, nullptr, nx, ny, nz, 0, 1.f, s)) != cudaSuccess) return e;
+    const unsigned tb = (unsigned)(nx + ny + nz + 31) / 32;
+    if ((e = launch_chained(twiddle_kernel, dim3(tb), dim3(32), 0, s, tw, nx, ny, nz)) != cudaSuccess) return e;
+    if ((e = dft<0, true, false>(W, tw, u, nullptr, nx, ny, nz, 0, 1.f, s)) != cudaSuccess) return e;
+    if ((e = dft<1, false, false>(W, tw, nullptr, nullptr, nx, ny, nz, 0, 1.f, s)) != cudaSuccess) return e;
+    if ((e = dft<2, false, false>(W, tw, nullptr, nullptr, nx, ny, nz, 0, 1.f, s)) != cudaSuccess) return e;
     const long long pb = (N + kThreads - 1) / kThreads;
-    project_modes_kernel<<<(unsigned)(pb < 4096 ? pb : 4096), kThreads, 0, s>>>(W, tw, nx, ny, nz);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = dft<2>(W, tw, nullptr, nullptr, nx, ny, nz, 1, 1.f, s)) != cudaSuccess) return e;
-    if ((e = dft<1>(W, tw, nullptr, nullptr, nx, ny, nz, 1, 1.f, s)) != cudaSuccess) return e;
-    return dft<0>(W, tw, nullptr, u, nx, ny, nz, 1, (float)(1.0 / (double)N), s);
+    e = launch_chained(project_modes_kernel, dim3((unsigned)(pb < 4096 ? pb : 4096)), dim3(kThreads), 0, s, W, (const float2*)tw, nx,
+                       ny, nz);
+    if (e != cudaSuccess) return e;
+    if ((e = dft<2, false, false>(W, tw, nullptr, nullptr, nx, ny, nz, 1, 1.f, s)) != cudaSuccess) return e;
+    if ((e = dft<1, false, false>(W, tw, nullptr, nullptr, nx, ny, nz, 1, 1.f, s)) != cudaSuccess) return e;
+    return dft<0, false, true>(W, tw, nullptr, u, nx, ny, nz, 1, (float)(1.0 / (double)N), s);
 }
 
 size_t project_workspace_bytes(int nx, int ny, int nz) { return proj::workspace_bytes(nx, ny, nz); }
