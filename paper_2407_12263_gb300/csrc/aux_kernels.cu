@@ -203,9 +203,13 @@ cudaError_t launch_moments(const Params& P, int scheme, int z0, int nzs, const v
 // populations. sum phi is the exact integer sum of the fixed-point phi values (64-bit), so it
 // reports conservation bit for bit; the other two accumulate in FP64. Grid-stride per thread,
 // warp shuffle, shared memory per block, one partial triple per block (the integer held in the
-// bits of the first double); a single block then sums the partials in a fixed order.
+// bits of the first double); a single block then sums the partials in a fixed order. Bound by the
+// stencil's loads: 71 us at 128^3 FP32, where one read of the state takes 47; it was 91 with a
+// second pass over the cell's own populations one by one, a 64-bit division per cell and a last wave
+// of blocks that left a third of the chip idle.
 // ---------------------------------------------------------------------------------------
 constexpr int kRedThreads = 256;
+constexpr int kMassBlocks = 4;  // of mass_kernel per SM
 
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {
@@ -236,7 +240,7 @@ __device__ __forceinline__ void block_sum(long long& s, double (&v)[2]) {
     }
 }
 
-template <int Q, int S>
+template <int Q, int S, bool WALLS>
 __global__ void __launch_bounds__(kRedThreads)
 mass_kernel(const Params P, const void* __restrict__ fg, double* __restrict__ partials) {
     long long phi_sum = 0, bad_sum = 0;
@@ -246,25 +250,34 @@ mass_kernel(const Params P, const void* __restrict__ fg, double* __restrict__ pa
     // of its FP32 rate); mass_finish scales them by 2^-60
     for (long long c = (long long)blockIdx.x * kRedThreads + threadIdx.x; c < P.N;
          c += (long long)gridDim.x * kRedThreads) {
-        const int z = (int)(c / P.nxy);
-        const int r = (int)(c - (long long)z * P.nxy);
+        const int z = (int)c / P.nxy, r = (int)c - z * P.nxy;  // c < N < 2^31
         const int y = r / P.nx, x = r - y * P.nx;
         const Nbr nb = make_nbr(P, x, y, z);
         float fb[Q], gb[Q];
         int phi_fx;
-        pull<Q, false, S, true>(P, fg, (int)c, nb, fb, gb, phi_fx, make_wall_side(P, x, y, z));
+        pull<Q, false, S, WALLS>(P, fg, (int)c, nb, fb, gb, phi_fx, WALLS ? make_wall_side(P, x, y, z) : WallSide{});
         const double q = (double)phi_fx;
         phi_sum += phi_fx;
         acc[0] += q * q;
-        int bad = 0;
+        // 0 times a finite value adds nothing, 0 times any other is NaN: the cell is looked at again then
         const float2 m0 = __ldg(moment_plane(fg) + c);
-        bad += !isfinite(m0.x);
+        float2 zero = make_float2(m0.x * 0.f, 0.f);
 #pragma unroll
-        for (int i = 1; i < Q; ++i) {
-            const float2 v = Store<S>::load(pop_ptr<Q, S>(fg, P.N, i, c), P);
-            bad += !isfinite(v.x) + !isfinite(v.y);
+        for (int k = 0; k < Lat<Q>::kPairs; ++k) {
+            const typename Store<S>::Word w = __ldg(pair_plane<S>(fg, P.N, k) + c);
+            zero = __ffma2_rn(Store<S>::cvt(Store<S>::lo(w)), make_float2(0.f, 0.f), zero);
+            zero = __ffma2_rn(Store<S>::cvt(Store<S>::hi(w)), make_float2(0.f, 0.f), zero);
         }
-        bad_sum += bad;
+        if (!(zero.x + zero.y == 0.f)) {
+            int bad = !isfinite(m0.x);
+#pragma unroll 1
+            for (int k = 0; k < Lat<Q>::kPairs; ++k) {
+                const typename Store<S>::Word w = __ldg(pair_plane<S>(fg, P.N, k) + c);
+                const float2 i = Store<S>::cvt(Store<S>::lo(w)), j = Store<S>::cvt(Store<S>::hi(w));
+                bad += !isfinite(i.x) + !isfinite(i.y) + !isfinite(j.x) + !isfinite(j.y);
+            }
+            bad_sum += bad;
+        }
     }
     acc[1] = (double)bad_sum;
     block_sum(phi_sum, acc);
@@ -368,9 +381,23 @@ int mass_partials_needed(const Params& P) {
     return (int)(blocks < 1024 ? blocks : 1024);
 }
 
+// At most `most` blocks, and no more than the SMs hold at once: threads stride over the cells, so one wave
+// of blocks leaves none idle at its end.
+static int wave_blocks(int most, int per_sm) {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return most;
+    return most < sms * per_sm ? most : sms * per_sm;
+}
+
 cudaError_t launch_mass(const Params& P, const void* fg, double* partials, int n_partials, double* result,
                         cudaStream_t s) {
-#define LBM_MASS(Q, S) mass_kernel<Q, S><<<n_partials, kRedThreads, 0, s>>>(P, fg, partials)
+#define LBM_MASS(Q, S)                                                                    \
+    do {                                                                                  \
+        if (P.walls) mass_kernel<Q, S, true><<<blocks, kRedThreads, 0, s>>>(P, fg, partials); \
+        else mass_kernel<Q, S, false><<<blocks, kRedThreads, 0, s>>>(P, fg, partials);    \
+    } while (0)
+    const int blocks = wave_blocks(n_partials, kMassBlocks);
     if (P.Q == 9) {
         if (P.storage == STORE_F16) LBM_MASS(9, STORE_F16);
         else if (P.storage == STORE_BF16) LBM_MASS(9, STORE_BF16);
@@ -381,7 +408,7 @@ cudaError_t launch_mass(const Params& P, const void* fg, double* partials, int n
         else LBM_MASS(19, STORE_F32);
     }
 #undef LBM_MASS
-    mass_finish<<<1, kRedThreads, 0, s>>>(partials, n_partials, P.rho2_d, P.drho_d, result);
+    mass_finish<<<1, kRedThreads, 0, s>>>(partials, blocks, P.rho2_d, P.drho_d, result);
     return cudaGetLastError();
 }
 
@@ -468,6 +495,8 @@ struct DiagArgs {
 //    the band takes the FP64 distance and the correctly rounded square root;
 //  * the energy and pressure sums: FP32 per cell and over runs of 8 of a thread's cells, each run
 //    then added to FP64 sums (one FP64 add per 8 cells whatever the grid size).
+// Two blocks per SM in one wave, 32-bit cell indices: 68 us at 128^3 FP32 (104 with 1024 blocks, the last of
+// whose four waves was a third full, and 64-bit divisions); one read of the state takes 47.
 template <int Q, int SCHEME, bool GEN, int S>
 __global__ void __launch_bounds__(kRedThreads, 2)
 diag_kernel(const Params P, const void* __restrict__ fg, const float* __restrict__ phi_fd, const DiagArgs A,
@@ -486,8 +515,7 @@ diag_kernel(const Params P, const void* __restrict__ fg, const float* __restrict
         float s2f = -1.0f;
         float ux = 0.f, uy = 0.f, uz = 0.f;
         if (valid) {
-            const int z = (int)(c / P.nxy);
-            const int r = (int)(c - (long long)z * P.nxy);
+            const int z = (int)c / P.nxy, r = (int)c - z * P.nxy;  // c < N < 2^31
             const int y = r / P.nx, x = r - y * P.nx;
             Macro m;
             int phi_fx;
@@ -588,6 +616,7 @@ double axis_d2_host(int i, double c, int n, bool wall) {
 
 cudaError_t launch_diagnostics(const Params& P, int scheme, const void* fg, const float* phi_fd, const double* d2_axes,
                                double r_in, double r_out, void* partials, int n_blocks, double* result, cudaStream_t s) {
+    n_blocks = wave_blocks(n_blocks, 2);
     // bands of 1e-5 relative around r^2: far wider than the FP32 rounding of the axis terms and
     // their sum (outside, FP32 decides the comparison of the correctly rounded FP64 distance)
     auto band = [](double r, double& lo, double& hi) {
