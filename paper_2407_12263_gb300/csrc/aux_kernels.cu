@@ -311,6 +311,8 @@ mass_finish(const double* __restrict__ partials, int n, double rho2, double drho
 // state that launch_mass reports in result[3], without reading the moving populations.
 __global__ void __launch_bounds__(kRedThreads)
 phi_fixed_sum_kernel(const float2* __restrict__ plane0, long long N, double* __restrict__ partials) {
+    chain_begin();
+    chain_next();
     long long s = 0;
     for (long long c = (long long)blockIdx.x * kRedThreads + threadIdx.x; c < N; c += (long long)gridDim.x * kRedThreads)
         s += __float_as_int(__ldg(plane0 + c).y);
@@ -321,6 +323,7 @@ phi_fixed_sum_kernel(const float2* __restrict__ plane0, long long N, double* __r
 
 __global__ void __launch_bounds__(kRedThreads)
 phi_fixed_finish(const double* __restrict__ partials, int n, double* __restrict__ result) {
+    chain_begin();
     long long s = 0;
     for (int b = threadIdx.x; b < n; b += kRedThreads) s += __double_as_longlong(partials[3 * b]);
     double unused[2] = {0.0, 0.0};
@@ -330,9 +333,9 @@ phi_fixed_finish(const double* __restrict__ partials, int n, double* __restrict_
 
 cudaError_t launch_phi_fixed_sum(const Params& P, const void* fg, double* partials, int n_partials, double* result,
                                  cudaStream_t s) {
-    phi_fixed_sum_kernel<<<n_partials, kRedThreads, 0, s>>>(moment_plane(fg), P.N, partials);
-    phi_fixed_finish<<<1, kRedThreads, 0, s>>>(partials, n_partials, result);
-    return cudaGetLastError();
+    const cudaError_t e = launch_chained(phi_fixed_sum_kernel, dim3(n_partials), dim3(kRedThreads), 0, s, moment_plane(fg), P.N, partials);
+    if (e != cudaSuccess) return e;
+    return launch_chained(phi_fixed_finish, dim3(1), dim3(kRedThreads), 0, s, (const double*)partials, n_partials, result);
 }
 
 // Validation of host input staged on the device: per block, the number of values outside

@@ -345,6 +345,8 @@ template <int F, bool BALANCE>
 __global__ void __launch_bounds__(128) coarse_phi_kernel(float2* __restrict__ plane0, int nx, int ny, int nz, const Balance B,
                                                          float* __restrict__ out) {
     __shared__ long long s_qr[2];
+    chain_begin();
+    chain_next();
     if (BALANCE) balance_of(B, s_qr);
     const int lane = threadIdx.x;
     const int x = blockIdx.x * 32 + lane;
@@ -403,8 +405,8 @@ template <int F>
 static void coarse_phi_f(const Params& P, void* fg, const RestartSums* sums, float* out, cudaStream_t s) {
     const dim3 block(32, 4), grid((P.nx + 31) / 32, (P.ny / F + 3) / 4, P.nz / F);
     const Balance B = balance_of_restart(P, sums);
-    if (sums) coarse_phi_kernel<F, true><<<grid, block, 0, s>>>(moment_plane(fg), P.nx, P.ny, P.nz, B, out);
-    else coarse_phi_kernel<F, false><<<grid, block, 0, s>>>(moment_plane(fg), P.nx, P.ny, P.nz, B, out);
+    (void)launch_chained(sums ? coarse_phi_kernel<F, true> : coarse_phi_kernel<F, false>, grid, block, 0, s, moment_plane(fg), P.nx,
+                         P.ny, P.nz, B, out);
 }
 
 cudaError_t launch_coarse_phi(const Params& P, void* fg, int factor, const RestartSums* sums, float* out, cudaStream_t s) {
@@ -487,6 +489,8 @@ __device__ __forceinline__ float trilinear(const float* __restrict__ q, const Co
 // The upsampled phi of every cell, the first pass of the restart, clamped to [-1, 1.5], the range
 // lbm_init_fields accepts, so that its fixed-point value stays in range whatever the prediction holds.
 __global__ void phi_fine_kernel(const Params P, const float* __restrict__ coarse, int f, float* __restrict__ phi) {
+    chain_begin();
+    chain_next();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
@@ -575,6 +579,7 @@ __global__ void __launch_bounds__(128)
 restart_kernel(const Params P, const float* __restrict__ coarse, const float* __restrict__ phi_fine, int f, float p0,
                void* __restrict__ fg, unsigned long long* __restrict__ slots, int n_slots) {
     __shared__ long long s_sum[4];
+    chain_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     int v = 0;
@@ -595,8 +600,9 @@ cudaError_t launch_restart(const Params& P, const float* coarse, int factor, dou
     cudaError_t e = cudaMemsetAsync(sums.slots, 0, sums.n_slots * sizeof(*sums.slots), s);
     if (e != cudaSuccess) return e;
     const dim3 block(32, 4), grid((P.nx + 31) / 32, (P.ny + 3) / 4, P.nz);
-    phi_fine_kernel<<<grid, block, 0, s>>>(P, coarse, factor, phi_fine);
-#define LBM_RESTART(Q, S) restart_kernel<Q, S><<<grid, block, 0, s>>>(P, coarse, phi_fine, factor, (float)p0, fg, sums.slots, sums.n_slots)
+    if ((e = launch_chained(phi_fine_kernel, grid, block, 0, s, P, coarse, factor, phi_fine)) != cudaSuccess) return e;
+#define LBM_RESTART(Q, S) \
+    e = launch_chained(restart_kernel<Q, S>, grid, block, 0, s, P, coarse, (const float*)phi_fine, factor, (float)p0, fg, sums.slots, sums.n_slots)
     if (P.Q == 9) {
         if (P.storage == STORE_F16) LBM_RESTART(9, STORE_F16);
         else if (P.storage == STORE_BF16) LBM_RESTART(9, STORE_BF16);
@@ -607,7 +613,7 @@ cudaError_t launch_restart(const Params& P, const float* coarse, int factor, dou
         else LBM_RESTART(19, STORE_F32);
     }
 #undef LBM_RESTART
-    return cudaGetLastError();
+    return e;
 }
 
 __device__ __forceinline__ double warp_sum_jm(double v) {
@@ -627,10 +633,12 @@ constexpr int kJumpThreads = 256;
 __global__ void __launch_bounds__(kJumpThreads)
 jump_measures_kernel(const float* __restrict__ start, const float* __restrict__ pred, int ncx, int ncy, int ncz,
                      int walls, double* __restrict__ out) {
+    chain_begin();
+    chain_next();
     const long long nc = (long long)ncx * ncy * ncz;
     double acc[3] = {0.0, 0.0, 0.0}, umax = 0.0;
     for (long long l = (long long)blockIdx.x * kJumpThreads + threadIdx.x; l < nc; l += (long long)gridDim.x * kJumpThreads) {
-        const int x = (int)(l % ncx), y = (int)((l / ncx) % ncy), z = (int)(l / ((long long)ncx * ncy));
+        const int row = (int)l / ncx, x = (int)l - row * ncx, z = row / ncy, y = row - z * ncy;  // nc < 2^31
         auto idx = [&](int xx, int yy, int zz) { return ((long long)zz * ncy + yy) * ncx + xx; };
         auto nb = [](int i, int d, int n, bool wall) { return wall ? min(max(i + d, 0), n - 1) : (i + d + n) % n; };
         const float ps = __ldg(start + l), pp = __ldg(pred + l);
@@ -681,13 +689,14 @@ cudaError_t launch_jump_measures(const float* start, const float* pred, int ncx,
                                  cudaStream_t s) {
     const long long nc = (long long)ncx * ncy * ncz;
     const long long blocks = (nc + kJumpThreads - 1) / kJumpThreads;
-    jump_measures_kernel<<<(unsigned)(blocks < 1216 ? blocks : 1216), kJumpThreads, 0, s>>>(start, pred, ncx, ncy, ncz,
-                                                                                           walls, out);
-    return cudaGetLastError();
+    return launch_chained(jump_measures_kernel, dim3((unsigned)(blocks < 1216 ? blocks : 1216)), dim3(kJumpThreads), 0, s, start, pred,
+                          ncx, ncy, ncz, walls, out);
 }
 
 __global__ void normalize_kernel(const float* __restrict__ x, float* __restrict__ y, long long n, float m0, float m1,
                                  float m2, float m3, float m4, float s0, float s1, float s2, float s3, float s4, int dir) {
+    chain_begin();
+    chain_next();
     const float mean[5] = {m0, m1, m2, m3, m4}, sd[5] = {s0, s1, s2, s3, s4};
     const int c = blockIdx.y;
     const float m = mean[c], d = sd[c];
@@ -698,15 +707,16 @@ __global__ void normalize_kernel(const float* __restrict__ x, float* __restrict_
 }
 
 cudaError_t launch_normalize(const float* x, float* y, long long n, const float* ms, int dir, cudaStream_t s) {
-    normalize_kernel<<<dim3(cell_blocks(n), 5), 256, 0, s>>>(x, y, n, ms[0], ms[1], ms[2], ms[3], ms[4], ms[5], ms[6], ms[7],
-                                                            ms[8], ms[9], dir);
-    return cudaGetLastError();
+    return launch_chained(normalize_kernel, dim3(cell_blocks(n), 5), dim3(256), 0, s, x, y, n, ms[0], ms[1], ms[2], ms[3], ms[4],
+                          ms[5], ms[6], ms[7], ms[8], ms[9], dir);
 }
 
 // sum |a - b| over n values in FP64: per block, then the blocks by one block, each in a fixed order.
 __global__ void __launch_bounds__(kJumpThreads) l1_kernel(const float* __restrict__ a, const float* __restrict__ b, long long n,
                                                          double* __restrict__ out) {
     __shared__ double red[kJumpThreads / 32];
+    chain_begin();
+    chain_next();
     double acc = 0.0;
     for (long long i = (long long)blockIdx.x * kJumpThreads + threadIdx.x; i < n; i += (long long)gridDim.x * kJumpThreads)
         acc += fabs((double)__ldg(a + i) - (double)__ldg(b + i));
@@ -721,6 +731,8 @@ __global__ void __launch_bounds__(kJumpThreads) l1_kernel(const float* __restric
 }
 __global__ void __launch_bounds__(kJumpThreads) l1_finish(const double* __restrict__ part, int n, double* __restrict__ out) {
     __shared__ double red[kJumpThreads / 32];
+    chain_begin();
+    chain_next();
     double acc = 0.0;
     for (int i = threadIdx.x; i < n; i += kJumpThreads) acc += part[i];
     acc = warp_sum_jm(acc);
@@ -736,9 +748,9 @@ __global__ void __launch_bounds__(kJumpThreads) l1_finish(const double* __restri
 cudaError_t launch_l1_difference(const float* a, const float* b, long long n, double* partials, int n_partials, double* out,
                                  cudaStream_t s) {
     const int blocks = (int)std::min<long long>((n + kJumpThreads - 1) / kJumpThreads, std::min(n_partials, 512));
-    l1_kernel<<<blocks, kJumpThreads, 0, s>>>(a, b, n, partials);
-    l1_finish<<<1, kJumpThreads, 0, s>>>(partials, blocks, out);
-    return cudaGetLastError();
+    const cudaError_t e = launch_chained(l1_kernel, dim3(blocks), dim3(kJumpThreads), 0, s, a, b, n, partials);
+    if (e != cudaSuccess) return e;
+    return launch_chained(l1_finish, dim3(1), dim3(kJumpThreads), 0, s, (const double*)partials, blocks, out);
 }
 
 }  // namespace lbm
