@@ -107,9 +107,10 @@ void drop_graphs(lbm_ctx* c) {
 // region with the most steps that still fits wins:
 //   side       40    64    96    128   184   216   256   304
 //   single     1.49  1.49  1.61  1.68  2.18  2.19  2.38  2.71   (difference-free, FP32)
-//   chosen     0.90  1.03  1.04  1.55  1.74  2.06  single single
+//   chosen     0.91  0.96  1.03  1.54  1.74  1.99  single single
 //   single     2.64  2.70  2.76  2.96  3.79  3.88  4.30  5.00   (finite-difference, two launches)
-//   chosen     1.16  1.35  1.42  1.93  2.30  2.96  3.40  single
+//   chosen     1.10  1.39  1.41  1.86  2.25  2.83  3.40  single
+// (single: blocks of whole rows; packed ones are up to 5% faster at sides of 184, 216 and 304)
 struct TileCost {
     int region;
     double fixed, per_step;
@@ -145,13 +146,11 @@ void plan_steps(lbm_ctx* c, int sms) {
         for (const TileCost& k : kTileDf) consider(k);
 }
 
-// n steps from buffer *cur, which ends as the one that holds the state. With `even` the launches are
-// even in number, so that *cur is what it was (n even).
-cudaError_t advance(const lbm_ctx* c, int n, bool even, int* cur, int* launches) {
+// n steps from buffer *cur, which ends as the one that holds the state.
+cudaError_t advance(const lbm_ctx* c, int n, int* cur, int* launches) {
     cudaError_t e = cudaSuccess;
     if (c->tile_steps > 1 && n > 1) {
-        int parts = (n + c->tile_steps - 1) / c->tile_steps;
-        if (even) parts = (parts + 1) / 2 * 2;
+        const int parts = (n + c->tile_steps - 1) / c->tile_steps;
         for (int k = 0; k < parts && e == cudaSuccess; ++k) {
             const int steps = n / parts + (k < n % parts);
             e = lbm::launch_tile_steps(c->P, c->scheme, c->tile_region, c->fg[*cur], c->fg[1 - *cur], steps, c->stream);
@@ -167,13 +166,16 @@ cudaError_t advance(const lbm_ctx* c, int n, bool even, int* cur, int* launches)
     return e;
 }
 
-// Captures graph_steps steps starting from buffer `start` (an even count returns to it).
+// Captures graph_steps steps starting from buffer `start`. An odd number of launches (several steps each)
+// ends in the other buffer, from where the other graph goes on: seven launches of 4 or 5 steps
+// for 32 steps of 64^2 take 30 us, eight of 4, which would return to the buffer, 33.
 int capture_graph(lbm_ctx* c, int start) {
     cudaGraph_t graph = nullptr;
     LBM_CUDA(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
     int launches = 0, cur = start;
-    cudaError_t e = advance(c, c->graph_steps, true, &cur, &launches);
+    cudaError_t e = advance(c, c->graph_steps, &cur, &launches);
     c->graph_launches = launches;
+    c->graph_flips = cur != start;
     cudaError_t e2 = cudaStreamEndCapture(c->stream, &graph);
     if (e == cudaSuccess) e = e2;
     if (e == cudaSuccess) e = cudaGraphInstantiate(&c->graph_exec[start], graph, 0);
@@ -564,11 +566,14 @@ int lbm_graph_prepare(lbm_ctx* c) {
     if (rc) return rc;
     if (c->graph_steps <= 0) return set_error(c, LBM_EINVAL, "the handle replays no graphs (graph_steps 0)");
     if (!c->initialised) return set_error(c, LBM_ESTATE, "no state: call lbm_init_phi first");
-    if (!c->graph_exec[c->cur]) {
-        rc = capture_graph(c, c->cur);
-        if (rc) return rc;
+    for (int start = c->cur, k = 0; k < 2; ++k, start = 1 - start) {
+        if (!c->graph_exec[start]) {
+            rc = capture_graph(c, start);
+            if (rc) return rc;
+        }
+        LBM_CUDA(c, cudaGraphUpload(c->graph_exec[start], c->stream));
+        if (!c->graph_flips) break;  // every replay starts from this buffer
     }
-    LBM_CUDA(c, cudaGraphUpload(c->graph_exec[c->cur], c->stream));
     LBM_CUDA(c, cudaStreamSynchronize(c->stream));
     return LBM_OK;
 }
@@ -588,11 +593,12 @@ int lbm_step(lbm_ctx* c, int n) {
             }
             LBM_CUDA(c, cudaGraphLaunch(c->graph_exec[c->cur], c->stream));
             c->launches += c->graph_launches;
-            n -= c->graph_steps;  // an even number of launches leaves the current buffer unchanged
+            n -= c->graph_steps;
+            if (c->graph_flips) c->cur = 1 - c->cur;
         }
     }
     int launches = 0;
-    const cudaError_t e = advance(c, n, false, &c->cur, &launches);
+    const cudaError_t e = advance(c, n, &c->cur, &launches);
     c->launches += launches;
     if (e != cudaSuccess) return set_error(c, LBM_ECUDA, "launching a step failed: %s", cudaGetErrorString(e));
     return LBM_OK;

@@ -29,6 +29,7 @@ struct lbm_ctx {
     int graph_steps;                  // steps per replayed CUDA graph (0 = none)
     cudaGraphExec_t graph_exec[2];    // graph of graph_steps steps starting from buffer 0 / 1
     int graph_launches;               // kernel launches of such a graph
+    bool graph_flips;                 // it ends in the other buffer
     int tile_region, tile_steps;      // D2Q9: steps per launch at most and their blocks' regions; 1: single steps
     bool batch_owned;      // a case of an lbm_batch: lbm_destroy leaves it to lbm_batch_destroy
     void* jump_ws;         // surrogate jumps: a backup state, then four coarse field arrays
