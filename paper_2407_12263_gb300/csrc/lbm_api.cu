@@ -146,11 +146,14 @@ void plan_steps(lbm_ctx* c, int sms) {
         for (const TileCost& k : kTileDf) consider(k);
 }
 
-// n steps from buffer *cur, which ends as the one that holds the state.
-cudaError_t advance(const lbm_ctx* c, int n, int* cur, int* launches) {
+// n steps from buffer *cur, which ends as the one that holds the state. With `parity` the launches are
+// even or odd in number as n is: a caller who captures an even number of steps may replay them, which
+// always start from the buffer they were captured from.
+cudaError_t advance(const lbm_ctx* c, int n, bool parity, int* cur, int* launches) {
     cudaError_t e = cudaSuccess;
     if (c->tile_steps > 1 && n > 1) {
-        const int parts = (n + c->tile_steps - 1) / c->tile_steps;
+        int parts = (n + c->tile_steps - 1) / c->tile_steps;
+        if (parity && ((parts ^ n) & 1)) ++parts;
         for (int k = 0; k < parts && e == cudaSuccess; ++k) {
             const int steps = n / parts + (k < n % parts);
             e = lbm::launch_tile_steps(c->P, c->scheme, c->tile_region, c->fg[*cur], c->fg[1 - *cur], steps, c->stream);
@@ -173,7 +176,7 @@ int capture_graph(lbm_ctx* c, int start) {
     cudaGraph_t graph = nullptr;
     LBM_CUDA(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
     int launches = 0, cur = start;
-    cudaError_t e = advance(c, c->graph_steps, &cur, &launches);
+    cudaError_t e = advance(c, c->graph_steps, false, &cur, &launches);
     c->graph_launches = launches;
     c->graph_flips = cur != start;
     cudaError_t e2 = cudaStreamEndCapture(c->stream, &graph);
@@ -598,7 +601,7 @@ int lbm_step(lbm_ctx* c, int n) {
         }
     }
     int launches = 0;
-    const cudaError_t e = advance(c, n, &c->cur, &launches);
+    const cudaError_t e = advance(c, n, cap != cudaStreamCaptureStatusNone, &c->cur, &launches);
     c->launches += launches;
     if (e != cudaSuccess) return set_error(c, LBM_ECUDA, "launching a step failed: %s", cudaGetErrorString(e));
     return LBM_OK;
