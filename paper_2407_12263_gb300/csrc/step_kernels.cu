@@ -108,7 +108,7 @@ static StepShape step_shape(const Params& P) {
     StepShape h;
     h.block = P.nx >= 128 ? dim3(128, 1, 1) : dim3(32, 4, 1);
     h.grid = dim3((P.nx + h.block.x - 1) / h.block.x, (P.ny + h.block.y - 1) / h.block.y, P.nz);
-    const unsigned blocks = (unsigned)((P.nxy + kStepThreads - 1) / kStepThreads);
+    const unsigned blocks = ((unsigned)P.nxy + kStepThreads - 1) / kStepThreads;
     h.form = P.nx > 1 && blocks < h.grid.x * h.grid.y ? PACKED : WHOLE;
     if (P.Q == 19 && P.storage != STORE_F32 && P.N >= (1ll << 29)) h.form = WIDE;
     h.d = RowDiv{0u, 0};
