@@ -310,19 +310,19 @@ mass_finish(const double* __restrict__ partials, int n, double rho2, double drho
 // faces in integer amounts that cancel in pairs, so this equals the sum over the propagated
 // state that launch_mass reports in result[3], without reading the moving populations.
 __global__ void __launch_bounds__(kRedThreads)
-phi_fixed_sum_kernel(const float2* __restrict__ plane0, long long N, double* __restrict__ partials) {
+phi_fixed_sum_kernel(const float2* plane0, long long N, double* __restrict__ partials) {
     chain_begin();
     chain_next();
     long long s = 0;
     for (long long c = (long long)blockIdx.x * kRedThreads + threadIdx.x; c < N; c += (long long)gridDim.x * kRedThreads)
-        s += __float_as_int(__ldg(plane0 + c).y);
+        s += __float_as_int(plane0[c].y);
     double unused[2] = {0.0, 0.0};
     block_sum(s, unused);
     if (threadIdx.x == 0) partials[3 * blockIdx.x] = __longlong_as_double(s);
 }
 
 __global__ void __launch_bounds__(kRedThreads)
-phi_fixed_finish(const double* __restrict__ partials, int n, double* __restrict__ result) {
+phi_fixed_finish(const double* partials, int n, double* __restrict__ result) {
     chain_begin();
     long long s = 0;
     for (int b = threadIdx.x; b < n; b += kRedThreads) s += __double_as_longlong(partials[3 * b]);

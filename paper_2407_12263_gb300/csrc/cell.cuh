@@ -130,7 +130,7 @@ __device__ __forceinline__ T* at_bytes(T* p, unsigned bytes) {
 // this cell's value) with one rounding; a difference a - b in the flux is written -(b - a),
 // which is the same number.
 template <int Q, bool WITH_F, int S, bool WALLS = false, bool RAW = false, bool NARROW = false>
-__device__ __forceinline__ void pull(const Params& P, const void* __restrict__ state, int c, const Nbr& nb,
+__device__ __forceinline__ void pull(const Params& P, const void* state, int c, const Nbr& nb,
                                      float (&fb)[Q], float (&gb)[Q], int& phi_fx,
                                      const WallSide& ws = WallSide{}) {
     using St = Store<S>;
@@ -162,7 +162,7 @@ __device__ __forceinline__ void pull(const Params& P, const void* __restrict__ s
                 qm = pw + c + ((int)im - c);
                 qp = pw + c + ((int)ip - c);
             }
-            const typename St::Word vm = __ldg(qm), v0 = __ldg(q0), vp = __ldg(qp);
+            const typename St::Word vm = *qm, v0 = *q0, vp = *qp;
             rmi = St::lo(vm);
             rpj = St::hi(vm);
             r0i = St::lo(v0);
@@ -195,8 +195,8 @@ __device__ __forceinline__ void pull(const Params& P, const void* __restrict__ s
             df += ei.x + ej.x;
         }
     }
-    const float2 m0 = NARROW ? __ldg(at_bytes(moment_plane(state), (unsigned)c * (unsigned)sizeof(float2)))
-                             : St::kUnsignedIndex ? __ldg(moment_plane(state) + (unsigned)c) : __ldg(moment_plane(state) + c);
+    const float2 m0 = NARROW ? *at_bytes(moment_plane(state), (unsigned)c * (unsigned)sizeof(float2))
+                             : St::kUnsignedIndex ? moment_plane(state)[(unsigned)c] : moment_plane(state)[c];
     phi_fx = (int)((unsigned int)__float_as_int(m0.y) + dphi);
     gb[0] = __int2float_rn((int)((unsigned int)phi_fx - (unsigned int)P.phi_ref_fx)) * kPhiFxInvF;
     if (WITH_F) fb[0] = m0.x + df * St::kInvF;
@@ -329,11 +329,11 @@ __device__ __forceinline__ void fd_term(int i, float v, float& gx, float& gy, fl
 }
 
 template <int Q>
-__device__ __forceinline__ void fd_gradient(const float* __restrict__ phi, int c, const Nbr& nb,
+__device__ __forceinline__ void fd_gradient(const float* phi, int c, const Nbr& nb,
                                             float& gx, float& gy, float& gz) {
     gx = gy = gz = 0.f;
 #pragma unroll
-    for (int i = 1; i < Q; ++i) fd_term<Q>(i, __ldg(phi + c + link_offset<Q>(nb, i, +1)), gx, gy, gz);
+    for (int i = 1; i < Q; ++i) fd_term<Q>(i, phi[c + link_offset<Q>(nb, i, +1)], gx, gy, gz);
     gx *= 3.f;
     gy *= 3.f;
     gz *= 3.f;
@@ -440,8 +440,8 @@ __device__ __forceinline__ void collide(const Params& P, const Macro& m, float (
 // post-collision pairs into fg_out. The single-case step kernel and the batched kernel both run
 // this, so a case gives the same bits whichever of them advances it.
 template <int Q, int SCHEME, bool GEN, int S, bool NARROW = false>
-__device__ __forceinline__ void step_cell(const Params& P, const void* __restrict__ fg_in, void* __restrict__ fg_out,
-                                          const float* __restrict__ phi_fd, int x, int y, int z) {
+__device__ __forceinline__ void step_cell(const Params& P, const void* fg_in, void* __restrict__ fg_out,
+                                          const float* phi_fd, int x, int y, int z) {
     const Nbr nb = make_nbr(P, x, y, z);
     const int c = (z * P.ny + y) * P.nx + x;
     const WallSide ws = GEN ? make_wall_side(P, x, y, z) : WallSide{};

@@ -9,6 +9,13 @@
 // to 80^3 in both schemes, FP32 and FP16, 1.01 to 1.21 times faster). chain_next() stands before a step's
 // stores: said at the start of a block, the next grid's first blocks take what slots are free and the
 // rest come unevenly to the SMs (304^2 15% slower than plain launches).
+//
+// Such a kernel is alive while the one before it still writes what it will read. It therefore loads with
+// ordinary loads through pointers without __restrict__, which the wait orders: __ldg, and the loads of a
+// `const T* __restrict__` parameter that the compiler turns into it, are for data that nobody writes in
+// the kernel's lifetime, may be moved above the wait, and go through a cache that need not see the
+// writes. (The same holds for a __restrict__ pointer of a kernel that only reads through it.) Ordinary
+// loads cost nothing: see the figures of step_shape, which are the same with either.
 #pragma once
 
 #include <cuda_runtime.h>

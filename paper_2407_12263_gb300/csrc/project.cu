@@ -68,8 +68,8 @@ __global__ void twiddle_kernel(float2* tw, int nx, int ny, int nz) {
 // zero imaginary parts add nothing to the sums and are left out. REAL_OUT (pass along x only): write
 // scale times the real part to [3][N] instead of W, and sum nothing else.
 template <int AXIS, bool REAL_IN, bool REAL_OUT>
-__global__ void __launch_bounds__(kThreads) dft_kernel(float2* __restrict__ W, const float2* __restrict__ tw_axis,
-                                                       const float* __restrict__ in_real, float* __restrict__ out_real,
+__global__ void __launch_bounds__(kThreads) dft_kernel(float2* W, const float2* tw_axis,
+                                                       const float* in_real, float* out_real,
                                                        int nx, int ny, int nz, int inverse, float scale) {
     extern __shared__ float2 sm[];
     const int n = AXIS == 0 ? nx : AXIS == 1 ? ny : nz;
@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(kThreads) dft_kernel(float2* __restrict__ W, c
 }
 
 // U <- U - s (s . U) / |s|^2 for every mode (kx, ky, kz); s_a = sin(2 pi k_a / n_a) = -Im w_a[k_a].
-__global__ void project_modes_kernel(float2* __restrict__ W, const float2* __restrict__ tw, int nx, int ny, int nz) {
+__global__ void project_modes_kernel(float2* W, const float2* tw, int nx, int ny, int nz) {
     chain_begin();
     chain_next();
     const long long N = (long long)nx * ny * nz;

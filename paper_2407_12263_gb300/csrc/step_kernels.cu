@@ -64,8 +64,7 @@ constexpr bool narrow_form(int form) { return Q == 19 && S != STORE_F32 && form 
 
 template <int Q, int SCHEME, bool GEN, int S, int FORM>
 __global__ void __launch_bounds__(kStepThreads, (step_min_blocks<S>()))
-step_kernel(const Params P, const void* __restrict__ fg_in, void* __restrict__ fg_out,
-            const float* __restrict__ phi_fd, const RowDiv d) {
+step_kernel(const Params P, const void* fg_in, void* __restrict__ fg_out, const float* phi_fd, const RowDiv d) {
     chain_begin();
     int x, y, z;
     if (!own_cell<FORM == PACKED>(P, d, x, y, z)) return;
@@ -75,7 +74,7 @@ step_kernel(const Params P, const void* __restrict__ fg_in, void* __restrict__ f
 // Finite-difference variant, pass 1: the propagated phi (held as phi - phi_ref), one FP32 plane.
 template <int Q, int S, bool WALLS, int FORM>
 __global__ void __launch_bounds__(kStepThreads, LBM_STEP_MINB)
-fd_phi_kernel(const Params P, const void* __restrict__ fg_in, float* __restrict__ phi, const RowDiv d) {
+fd_phi_kernel(const Params P, const void* fg_in, float* __restrict__ phi, const RowDiv d) {
     chain_begin();
     int x, y, z;
     if (!own_cell<FORM == PACKED>(P, d, x, y, z)) return;

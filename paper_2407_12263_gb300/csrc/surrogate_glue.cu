@@ -342,7 +342,7 @@ __device__ __forceinline__ int balanced(int phi_fx, long long c, const long long
 // with shuffles. With the factor known the loads of eight rows are in flight at once: 128^3 at F = 2
 // 18 -> 6 us, 9 us with the balance (8.6 us as a pass of its own).
 template <int F, bool BALANCE>
-__global__ void __launch_bounds__(128) coarse_phi_kernel(float2* __restrict__ plane0, int nx, int ny, int nz, const Balance B,
+__global__ void __launch_bounds__(128) coarse_phi_kernel(float2* plane0, int nx, int ny, int nz, const Balance B,
                                                          float* __restrict__ out) {
     __shared__ long long s_qr[2];
     chain_begin();
@@ -477,18 +477,18 @@ __device__ __forceinline__ Corners corners(int ncx, int ncy, const Axis& X, cons
 }
 
 // Trilinear interpolation of q at the corners: along x, then y, then z
-__device__ __forceinline__ float trilinear(const float* __restrict__ q, const Corners& c) {
+__device__ __forceinline__ float trilinear(const float* q, const Corners& c) {
     auto lerp = [](float u, float v, float t) { return fmaf(t, v - u, u); };
-    const float c00 = lerp(__ldg(q + c.o[0]), __ldg(q + c.o[1]), c.tx);
-    const float c01 = lerp(__ldg(q + c.o[2]), __ldg(q + c.o[3]), c.tx);
-    const float c10 = lerp(__ldg(q + c.o[4]), __ldg(q + c.o[5]), c.tx);
-    const float c11 = lerp(__ldg(q + c.o[6]), __ldg(q + c.o[7]), c.tx);
+    const float c00 = lerp(q[c.o[0]], q[c.o[1]], c.tx);
+    const float c01 = lerp(q[c.o[2]], q[c.o[3]], c.tx);
+    const float c10 = lerp(q[c.o[4]], q[c.o[5]], c.tx);
+    const float c11 = lerp(q[c.o[6]], q[c.o[7]], c.tx);
     return lerp(lerp(c00, c01, c.ty), lerp(c10, c11, c.ty), c.tz);
 }
 
 // The upsampled phi of every cell, the first pass of the restart, clamped to [-1, 1.5], the range
 // lbm_init_fields accepts, so that its fixed-point value stays in range whatever the prediction holds.
-__global__ void phi_fine_kernel(const Params P, const float* __restrict__ coarse, int f, float* __restrict__ phi) {
+__global__ void phi_fine_kernel(const Params P, const float* coarse, int f, float* __restrict__ phi) {
     chain_begin();
     chain_next();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -509,19 +509,19 @@ __global__ void phi_fine_kernel(const Params P, const float* __restrict__ coarse
 // any order). Bound by instructions: the arithmetic is written with the velocities' zero components,
 // and 16-bit restarts, which amplify a last bit, fix its roundings.
 template <int Q, int S>
-__device__ __forceinline__ int restart_cell(const Params& P, const float* __restrict__ coarse, const float* __restrict__ phi_fine,
+__device__ __forceinline__ int restart_cell(const Params& P, const float* coarse, const float* phi_fine,
                                             int f, float p0, void* __restrict__ fg, int x, int y, int z) {
     const int ncx = P.nx / f, ncy = P.ny / f, ncz = P.nz / f;
     const long long nc = (long long)ncx * ncy * ncz;
     // neighbours: periodic images, or across a wall the cell itself (so that the normal gradient
     // vanishes there); the grid holds fewer than 2^31 cells
     const Nbr nb = mirror_at_walls(make_nbr(P, x, y, z), make_wall_side(P, x, y, z));
-    const float* __restrict__ here = phi_fine + ((z * P.ny + y) * P.nx + x);
-    const float phi = __ldg(here);
+    const float* here = phi_fine + ((z * P.ny + y) * P.nx + x);
+    const float phi = *here;
     float gx = 0.f, gy = 0.f, gz = 0.f;
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
-        const float v = Lat<Q>::w(i) * __ldg(here + link_offset<Q>(nb, i, +1));
+        const float v = Lat<Q>::w(i) * here[link_offset<Q>(nb, i, +1)];
         gx += Lat<Q>::cx(i) * v;
         gy += Lat<Q>::cy(i) * v;
         gz += Lat<Q>::cz(i) * v;
@@ -576,7 +576,7 @@ __device__ __forceinline__ int restart_cell(const Params& P, const float* __rest
 
 template <int Q, int S>
 __global__ void __launch_bounds__(128)
-restart_kernel(const Params P, const float* __restrict__ coarse, const float* __restrict__ phi_fine, int f, float p0,
+restart_kernel(const Params P, const float* coarse, const float* phi_fine, int f, float p0,
                void* __restrict__ fg, unsigned long long* __restrict__ slots, int n_slots) {
     __shared__ long long s_sum[4];
     chain_begin();
@@ -631,7 +631,7 @@ __device__ __forceinline__ double warp_max_jm(double v) {
 constexpr int kJumpThreads = 256;
 
 __global__ void __launch_bounds__(kJumpThreads)
-jump_measures_kernel(const float* __restrict__ start, const float* __restrict__ pred, int ncx, int ncy, int ncz,
+jump_measures_kernel(const float* start, const float* pred, int ncx, int ncy, int ncz,
                      int walls, double* __restrict__ out) {
     chain_begin();
     chain_next();
@@ -641,20 +641,20 @@ jump_measures_kernel(const float* __restrict__ start, const float* __restrict__ 
         const int row = (int)l / ncx, x = (int)l - row * ncx, z = row / ncy, y = row - z * ncy;  // nc < 2^31
         auto idx = [&](int xx, int yy, int zz) { return ((long long)zz * ncy + yy) * ncx + xx; };
         auto nb = [](int i, int d, int n, bool wall) { return wall ? min(max(i + d, 0), n - 1) : (i + d + n) % n; };
-        const float ps = __ldg(start + l), pp = __ldg(pred + l);
+        const float ps = start[l], pp = pred[l];
         acc[0] += (double)pp;
         acc[1] += fabs((double)pp - (double)ps);
-        const double gx = 0.5 * ((double)__ldg(start + idx(nb(x, 1, ncx, walls & 1), y, z)) -
-                                 (double)__ldg(start + idx(nb(x, -1, ncx, walls & 1), y, z)));
-        const double gy = 0.5 * ((double)__ldg(start + idx(x, nb(y, 1, ncy, walls & 2), z)) -
-                                 (double)__ldg(start + idx(x, nb(y, -1, ncy, walls & 2), z)));
-        const double gz = 0.5 * ((double)__ldg(start + idx(x, y, nb(z, 1, ncz, walls & 4))) -
-                                 (double)__ldg(start + idx(x, y, nb(z, -1, ncz, walls & 4))));
+        const double gx = 0.5 * ((double)start[idx(nb(x, 1, ncx, walls & 1), y, z)] -
+                                 (double)start[idx(nb(x, -1, ncx, walls & 1), y, z)]);
+        const double gy = 0.5 * ((double)start[idx(x, nb(y, 1, ncy, walls & 2), z)] -
+                                 (double)start[idx(x, nb(y, -1, ncy, walls & 2), z)]);
+        const double gz = 0.5 * ((double)start[idx(x, y, nb(z, 1, ncz, walls & 4))] -
+                                 (double)start[idx(x, y, nb(z, -1, ncz, walls & 4))]);
         acc[2] += sqrt(gx * gx + gy * gy + gz * gz);
         double u2s = 0.0, u2p = 0.0;
 #pragma unroll
         for (int a = 1; a <= 3; ++a) {
-            const double us = __ldg(start + a * nc + l), up = __ldg(pred + a * nc + l);
+            const double us = start[a * nc + l], up = pred[a * nc + l];
             u2s += us * us;
             u2p += up * up;
         }
@@ -693,7 +693,7 @@ cudaError_t launch_jump_measures(const float* start, const float* pred, int ncx,
                           ncx, ncy, ncz, walls, out);
 }
 
-__global__ void normalize_kernel(const float* __restrict__ x, float* __restrict__ y, long long n, float m0, float m1,
+__global__ void normalize_kernel(const float* x, float* __restrict__ y, long long n, float m0, float m1,
                                  float m2, float m3, float m4, float s0, float s1, float s2, float s3, float s4, int dir) {
     chain_begin();
     chain_next();
@@ -712,14 +712,14 @@ cudaError_t launch_normalize(const float* x, float* y, long long n, const float*
 }
 
 // sum |a - b| over n values in FP64: per block, then the blocks by one block, each in a fixed order.
-__global__ void __launch_bounds__(kJumpThreads) l1_kernel(const float* __restrict__ a, const float* __restrict__ b, long long n,
+__global__ void __launch_bounds__(kJumpThreads) l1_kernel(const float* a, const float* b, long long n,
                                                          double* __restrict__ out) {
     __shared__ double red[kJumpThreads / 32];
     chain_begin();
     chain_next();
     double acc = 0.0;
     for (long long i = (long long)blockIdx.x * kJumpThreads + threadIdx.x; i < n; i += (long long)gridDim.x * kJumpThreads)
-        acc += fabs((double)__ldg(a + i) - (double)__ldg(b + i));
+        acc += fabs((double)a[i] - (double)b[i]);
     acc = warp_sum_jm(acc);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
@@ -729,7 +729,7 @@ __global__ void __launch_bounds__(kJumpThreads) l1_kernel(const float* __restric
         out[blockIdx.x] = acc;
     }
 }
-__global__ void __launch_bounds__(kJumpThreads) l1_finish(const double* __restrict__ part, int n, double* __restrict__ out) {
+__global__ void __launch_bounds__(kJumpThreads) l1_finish(const double* part, int n, double* __restrict__ out) {
     __shared__ double red[kJumpThreads / 32];
     chain_begin();
     chain_next();

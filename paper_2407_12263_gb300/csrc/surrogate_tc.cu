@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(kConvThreads, 2) conv_tc_kernel(const __grid_c
         float bias[MODE == kAdjoint ? 1 : kOut];
         if (MODE != kAdjoint)
 #pragma unroll
-            for (int ch = 0; ch < kOut; ++ch) bias[ch] = __ldg(A.bias + ch);
+            for (int ch = 0; ch < kOut; ++ch) bias[ch] = A.bias[ch];
         Walk walk(A.t);
         for (Column c; ok && walk.next(A.t, c);) {
             const int x = c.x0 + t % TX, y = c.y0 + t / TX;
@@ -486,12 +486,12 @@ __global__ void __launch_bounds__(kConvThreads, 2) conv_tc_kernel(const __grid_c
             auto fetch = [&](long long row, long long e) {
                 Extra f{};
                 if (!inside) return f;
-                if (MODE == kAdjoint) f.bits = __ldg(A.bits + row);
+                if (MODE == kAdjoint) f.bits = A.bits[row];
                 if (MODE == kPrediction || MODE == kLossGrad)
 #pragma unroll
                     for (int ch = 0; ch < kFieldChannels; ++ch) {
-                        f.x[ch] = __ldg(A.x + e + ch * vox);
-                        if (MODE == kLossGrad) f.t[ch] = __ldg(A.target + e + ch * vox);
+                        f.x[ch] = A.x[e + ch * vox];
+                        if (MODE == kLossGrad) f.t[ch] = A.target[e + ch * vox];
                     }
                 return f;
             };
@@ -826,7 +826,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_tc_kernel(const __grid_co
 // ---------------------------------------------------------------------------------------
 
 // FP16 copy of the fields x [B][5][vox], channels last and padded to 8.
-__global__ void pack_fields_kernel(const float* __restrict__ x, uint4* __restrict__ out, long long vox, int batch) {
+__global__ void pack_fields_kernel(const float* x, uint4* __restrict__ out, long long vox, int batch) {
     chain_begin();
     chain_next();
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < vox * batch; i += (long long)gridDim.x * blockDim.x) {
@@ -834,7 +834,7 @@ __global__ void pack_fields_kernel(const float* __restrict__ x, uint4* __restric
         const float* p = x + b * kFieldChannels * vox + (i - b * vox);
         float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int c = 0; c < kFieldChannels; ++c) v[c] = __ldg(p + c * vox);
+        for (int c = 0; c < kFieldChannels; ++c) v[c] = p[c * vox];
         __half2 h[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) h[c] = __floats2half2_rn(v[2 * c], v[2 * c + 1]);
@@ -901,7 +901,7 @@ __global__ void __launch_bounds__(kFinishThreads) grads_finish_kernel(const __gr
         for (int k = k0; k < k1; k += 20) {
             float v[20];
 #pragma unroll
-            for (int i = 0; i < 20; ++i) v[i] = __ldg(p + min(k + i, last) * 32);
+            for (int i = 0; i < 20; ++i) v[i] = p[min(k + i, last) * 32];
 #pragma unroll
             for (int i = 0; i < 20; ++i) acc += k + i < k1 ? v[i] : 0.f;
         }
@@ -925,7 +925,7 @@ __global__ void __launch_bounds__(kFinishThreads) grads_finish_kernel(const __gr
         for (int k = k0; k < k1; k += 10) {
             float4 v[10];
 #pragma unroll
-            for (int i = 0; i < 10; ++i) v[i] = __ldg(reinterpret_cast<const float4*>(p + (long long)min(k + i, last) * L.n));
+            for (int i = 0; i < 10; ++i) v[i] = *reinterpret_cast<const float4*>(p + (long long)min(k + i, last) * L.n);
 #pragma unroll
             for (int i = 0; i < 10; ++i)
                 if (k + i < k1) {

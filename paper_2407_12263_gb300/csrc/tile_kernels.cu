@@ -81,7 +81,7 @@ constexpr size_t tile_smem() {
 
 template <int R, int SCHEME, bool GEN, int S>
 __global__ void __launch_bounds__(R* R)
-tile_step_kernel(const Params P, const void* __restrict__ fg_in, void* __restrict__ fg_out, int steps) {
+tile_step_kernel(const Params P, const void* fg_in, void* __restrict__ fg_out, int steps) {
     using Word = typename Store<S>::Word;
     constexpr int n = R * R, kReach = SCHEME == SCHEME_FD ? 2 : 1;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -99,8 +99,8 @@ tile_step_kernel(const Params P, const void* __restrict__ fg_in, void* __restric
     chain_begin();
     if (!beyond) {
 #pragma unroll
-        for (int k = 0; k < Lat<Q9>::kPairs; ++k) words[k * n + c] = __ldg(pair_plane<S>(fg_in, P.N, k) + cell);
-        moments[c] = __ldg(moment_plane(fg_in) + cell);
+        for (int k = 0; k < Lat<Q9>::kPairs; ++k) words[k * n + c] = pair_plane<S>(fg_in, P.N, k)[cell];
+        moments[c] = moment_plane(fg_in)[cell];
     }
     const WallSide ws = GEN ? make_wall_side(P, x, y, 0) : WallSide{};
     const bool at_wall = GEN && (ws.xlo || ws.xhi || ws.ylo || ws.yhi);
