@@ -154,7 +154,16 @@ int lbm_init_fields(lbm_ctx *ctx, const double *phi0, const double *u0, const do
 
 /* Advance n >= 0 time steps (asynchronous on the handle's stream). Whole multiples of
  * opts.graph_steps are replayed from CUDA graphs the handle captures on first use; the rest
- * are launched directly. Both give bit-identical results. */
+ * are launched directly. Both give bit-identical results.
+ *
+ * lbm_step, lbm_coarse_fields and lbm_coarse_phi may be captured in a caller's CUDA graph, which then
+ * holds the address of the buffer that the state was in. It may be replayed whenever the state is in
+ * that buffer again. On a handle of which a call has been captured, as on one with the caller's
+ * buffers (lbm_create_ext) and on a case of a batch, the state changes its buffer with every step: what may
+ * stand between capture and replay, and between two replays, is any calls that make an even number
+ * of steps in all (whatever number each of them makes), initialisations and restarts, and surrogate jumps:
+ * accepted ones end in the buffer they began in, a rejected one counts as its k steps. A graph of an
+ * odd number of steps is replayed an even number of times. */
 int lbm_step(lbm_ctx *ctx, int n);
 
 /* Capture the step graph that lbm_step replays from the current state's buffer (and the one from the

@@ -145,6 +145,8 @@ typedef struct {
  *      exceeds relax_tol times the rate of step 3: a prediction whose phi, u and p do not fit
  *      together relaxes faster than the starting state does after the same restart;
  *   5. on rejection restore the starting state and advance it k steps with the LBM.
+ * Where lbm_step's contract on captured graphs has the state change its buffer with every step, an
+ * accepted jump ends in the buffer it began in, at the price of a copy of the state.
  * Synchronous. Needs a workspace of one more state buffer, four coarse field arrays and the
  * projection's scratch (lbm_project_workspace_bytes of the coarse grid): the
  * first jump on a handle allocates it (or lbm_surrogate_reserve, beforehand) and the handle keeps

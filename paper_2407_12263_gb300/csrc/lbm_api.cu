@@ -97,6 +97,7 @@ void drop_graphs(lbm_ctx* c) {
             cudaGraphExecDestroy(c->graph_exec[k]);
             c->graph_exec[k] = nullptr;
         }
+    c->graph_flips = false;
 }
 
 // How the steps of a D2Q9 grid are launched: several per launch (launch_tile_steps) where the regions
@@ -146,9 +147,8 @@ void plan_steps(lbm_ctx* c, int sms) {
         for (const TileCost& k : kTileDf) consider(k);
 }
 
-// n steps from buffer *cur, which ends as the one that holds the state. With `parity` the launches are
-// even or odd in number as n is: a caller who captures an even number of steps may replay them, which
-// always start from the buffer they were captured from.
+// n steps from buffer *cur, which ends as the one that holds the state. With `parity` (ctx_keeps_parity)
+// the launches are even or odd in number as n is.
 cudaError_t advance(const lbm_ctx* c, int n, bool parity, int* cur, int* launches) {
     cudaError_t e = cudaSuccess;
     if (c->tile_steps > 1 && n > 1) {
@@ -171,12 +171,13 @@ cudaError_t advance(const lbm_ctx* c, int n, bool parity, int* cur, int* launche
 
 // Captures graph_steps steps starting from buffer `start`. An odd number of launches (several steps each)
 // ends in the other buffer, from where the other graph goes on: seven launches of 4 or 5 steps
-// for 32 steps of 64^2 take 30 us, eight of 4, which would return to the buffer, 33.
+// for 32 steps of 64^2 take 30 us, eight of 4, which return to the buffer, 33. Those are captured where
+// the buffer has to follow the parity.
 int capture_graph(lbm_ctx* c, int start) {
     cudaGraph_t graph = nullptr;
     LBM_CUDA(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
     int launches = 0, cur = start;
-    cudaError_t e = advance(c, c->graph_steps, false, &cur, &launches);
+    cudaError_t e = advance(c, c->graph_steps, lbm::ctx_keeps_parity(c), &cur, &launches);
     c->graph_launches = launches;
     c->graph_flips = cur != start;
     cudaError_t e2 = cudaStreamEndCapture(c->stream, &graph);
@@ -188,6 +189,11 @@ int capture_graph(lbm_ctx* c, int start) {
         return set_error(c, LBM_ECUDA, "capturing the step graph failed: %s", cudaGetErrorString(e));
     }
     return LBM_OK;
+}
+
+// Graphs that end in the other buffer, captured before the buffer had to follow the parity.
+void drop_flipping_graphs(lbm_ctx* c) {
+    if (c->graph_flips && lbm::ctx_keeps_parity(c)) drop_graphs(c);
 }
 
 // The storage of the moving pairs (the FP16 scaling is a compile-time constant of Store<S>),
@@ -425,6 +431,17 @@ int lbm::ctx_check(lbm_ctx* c) { return check_ctx(c); }
 
 void lbm::ctx_drop_graphs(lbm_ctx* c) { drop_graphs(c); }
 
+bool lbm::ctx_keeps_parity(const lbm_ctx* c) { return c->captured || !c->own_fg || c->batch_owned; }
+
+void lbm::ctx_note_capture(lbm_ctx* c) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {
+        (void)cudaGetLastError();  // the legacy stream beside another's capture: the launch reports it
+        cap = cudaStreamCaptureStatusActive;
+    }
+    if (cap != cudaStreamCaptureStatusNone) c->captured = true;
+}
+
 int lbm::ctx_restart(lbm_ctx* c, int f, const float* coarse, double p0, const long long* before, void* fg, RestartSums* sums) {
     Params& P = c->P;
     const double w0d = p0 * 3.0;
@@ -569,6 +586,7 @@ int lbm_graph_prepare(lbm_ctx* c) {
     if (rc) return rc;
     if (c->graph_steps <= 0) return set_error(c, LBM_EINVAL, "the handle replays no graphs (graph_steps 0)");
     if (!c->initialised) return set_error(c, LBM_ESTATE, "no state: call lbm_init_phi first");
+    drop_flipping_graphs(c);
     for (int start = c->cur, k = 0; k < 2; ++k, start = 1 - start) {
         if (!c->graph_exec[start]) {
             rc = capture_graph(c, start);
@@ -588,7 +606,9 @@ int lbm_step(lbm_ctx* c, int n) {
     if (!c->initialised) return set_error(c, LBM_ESTATE, "lbm_step before lbm_init_phi");
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     LBM_CUDA(c, cudaStreamIsCapturing(c->stream, &cap));
+    if (cap != cudaStreamCaptureStatusNone) c->captured = true;
     if (c->graph_steps > 0 && cap == cudaStreamCaptureStatusNone) {
+        drop_flipping_graphs(c);
         while (n >= c->graph_steps) {
             if (!c->graph_exec[c->cur]) {
                 rc = capture_graph(c, c->cur);
@@ -601,7 +621,7 @@ int lbm_step(lbm_ctx* c, int n) {
         }
     }
     int launches = 0;
-    const cudaError_t e = advance(c, n, cap != cudaStreamCaptureStatusNone, &c->cur, &launches);
+    const cudaError_t e = advance(c, n, lbm::ctx_keeps_parity(c), &c->cur, &launches);
     c->launches += launches;
     if (e != cudaSuccess) return set_error(c, LBM_ECUDA, "launching a step failed: %s", cudaGetErrorString(e));
     return LBM_OK;

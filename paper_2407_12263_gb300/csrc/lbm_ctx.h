@@ -30,6 +30,7 @@ struct lbm_ctx {
     cudaGraphExec_t graph_exec[2];    // graph of graph_steps steps starting from buffer 0 / 1
     int graph_launches;               // kernel launches of such a graph
     bool graph_flips;                 // it ends in the other buffer
+    bool captured;                    // a caller's capture has recorded a call that holds a buffer's address
     int tile_region, tile_steps;      // D2Q9: steps per launch at most and their blocks' regions; 1: single steps
     bool batch_owned;      // a case of an lbm_batch: lbm_destroy leaves it to lbm_batch_destroy
     void* jump_ws;         // surrogate jumps: a backup state, then four coarse field arrays
@@ -59,6 +60,11 @@ int set_ctx_storage(lbm_ctx* c, int storage);
 int ctx_error(lbm_ctx* c, int code, const char* msg);
 int ctx_check(lbm_ctx* c);
 void ctx_drop_graphs(lbm_ctx* c);  // captured steps, after a change of parameters
+// Whether the buffer that holds the state follows the parity of the steps taken, because somebody holds
+// its address: a caller who has captured a call of the handle, who owns the buffers, or a batch.
+bool ctx_keeps_parity(const lbm_ctx* c);
+// To be called by what reads the state in launches alone, which a caller may capture.
+void ctx_note_capture(lbm_ctx* c);
 // The state lbm_init_fields builds from the coarse fields [5][nz/f][ny/f][nx/f] (device FP32: phi, u,
 // v, w, p) upsampled trilinearly, into the state buffer fg; p0 = the storage reference pressure. *sums
 // is what launch_balance (or launch_coarse_phi) then takes to set sum phi to *before (device).

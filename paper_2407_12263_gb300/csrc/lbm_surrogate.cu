@@ -15,6 +15,7 @@
 #include "../../include/lbm.h"
 #include "../../include/lbm_surrogate.h"
 #include "lbm_ctx.h"
+#include "storage.cuh"
 #include "surrogate.h"
 
 using lbm::net::kFieldChannels;
@@ -395,6 +396,7 @@ int lbm_coarse_fields(lbm_ctx* c, int f, float* out) {
         return lbm::ctx_error(c, LBM_EINVAL, "factor must divide nx, ny and nz, and out may not be NULL");
     if (!c->initialised) return lbm::ctx_error(c, LBM_ESTATE, "no state: call lbm_init_phi first");
     if (c->scheme != LBM_SCHEME_DIFFERENCE_FREE) return lbm::ctx_error(c, LBM_EINVAL, "coarse fields need the difference-free scheme");
+    lbm::ctx_note_capture(c);
     cudaError_t e = lbm::launch_coarsen(c->P, c->fg[c->cur], f, out, c->stream);
     if (e != cudaSuccess) return lbm::ctx_error(c, LBM_ECUDA, cudaGetErrorString(e));
     c->launches += 1;
@@ -407,6 +409,7 @@ int lbm_coarse_phi(lbm_ctx* c, int f, float* out) {
     if (!out || f < 1 || f > 32 || 32 % f || c->P.nx % f || c->P.ny % f || c->P.nz % f)
         return lbm::ctx_error(c, LBM_EINVAL, "factor must divide 32, nx, ny and nz, and out may not be NULL");
     if (!c->initialised) return lbm::ctx_error(c, LBM_ESTATE, "no state: call lbm_init_phi first");
+    lbm::ctx_note_capture(c);
     cudaError_t e = lbm::launch_coarse_phi(c->P, c->fg[c->cur], f, nullptr, out, c->stream);
     if (e != cudaSuccess) return lbm::ctx_error(c, LBM_ECUDA, cudaGetErrorString(e));
     c->launches += 1;
@@ -601,6 +604,12 @@ int lbm_surrogate_jump(lbm_ctx* c, lbm_net* n, int f, const float mean_std[10], 
     c->version += 1;
     if (accept) {
         c->cur = 1 - c->cur;
+        if (lbm::ctx_keeps_parity(c)) {  // back to the buffer that the jump began in
+            rc = cu(cudaMemcpyAsync(start, c->fg[c->cur], lbm::state_bytes(c->P.Q, c->P.N, c->P.storage), cudaMemcpyDeviceToDevice, c->stream));
+            if (rc) return rc;
+            c->cur = 1 - c->cur;
+            if ((rc = cu(cudaStreamSynchronize(c->stream)))) return rc;
+        }
     } else {  // 5. fallback
         if (c->P.w0d != saved_P.w0d) lbm::ctx_drop_graphs(c);
         c->P = saved_P;
