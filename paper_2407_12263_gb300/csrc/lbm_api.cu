@@ -18,6 +18,7 @@
 #include "diagnostics.h"
 #include "lbm_ctx.h"
 #include "lbm_internal.h"
+#include "step_plan.h"
 #include "storage.cuh"
 #include "surrogate.h"
 
@@ -100,63 +101,16 @@ void drop_graphs(lbm_ctx* c) {
     c->graph_flips = false;
 }
 
-// How the steps of a D2Q9 grid are launched: several per launch (launch_tile_steps) where the regions
-// of every tile fit the SMs at once, one block each, and that is faster than single steps. Costs are
-// microseconds on GB300, measured on square grids of 40 to 304 cells: a launch over regions of 16, 24
-// or 32 cells squared takes fixed + per_step * steps while blocks <= SMs (twice that for the larger
-// regions beyond), single steps a floor and a part that grows with the grid's side. The smallest
-// region with the most steps that still fits wins:
-//   side       40    64    96    128   184   216   256   304
-//   single     1.49  1.49  1.61  1.68  2.18  2.19  2.38  2.71   (difference-free, FP32)
-//   chosen     0.91  0.96  1.03  1.54  1.74  1.99  single single
-//   single     2.64  2.70  2.76  2.96  3.79  3.88  4.30  5.00   (finite-difference, two launches)
-//   chosen     1.10  1.39  1.41  1.86  2.25  2.83  3.40  single
-// (single: blocks of whole rows; packed ones are up to 5% faster at sides of 184, 216 and 304)
-struct TileCost {
-    int region;
-    double fixed, per_step;
-};
-constexpr TileCost kTileDf[] = {{16, 1.52, 0.66}, {24, 3.1, 0.90}};
-constexpr TileCost kTileFd[] = {{16, 1.9, 0.45}, {24, 2.6, 0.90}, {32, 3.7, 1.45}};
-
-void plan_steps(lbm_ctx* c, int sms) {
-    c->tile_region = 0;
-    c->tile_steps = 1;
-    const Params& P = c->P;
-    if (P.Q != 9) return;
-    const bool fd = c->scheme == LBM_SCHEME_FINITE_DIFFERENCE;
-    const double side = std::sqrt((double)P.N);
-    double best = fd ? std::max(2.65, 1.2 + 0.0125 * side) : std::max(1.48, 0.95 + 0.0058 * side);
-    auto consider = [&](const TileCost& k) {
-        for (int steps = 2; steps <= 8; ++steps) {
-            const int tile = k.region - 2 * steps * (fd ? 2 : 1);
-            if (tile < 4) break;
-            const long long blocks = (long long)((P.nx + tile - 1) / tile) * ((P.ny + tile - 1) / tile);
-            if (blocks > sms) break;
-            const double cost = k.fixed / steps + k.per_step;
-            if (cost < best) {
-                best = cost;
-                c->tile_region = k.region;
-                c->tile_steps = steps;
-            }
-        }
-    };
-    if (fd)
-        for (const TileCost& k : kTileFd) consider(k);
-    else
-        for (const TileCost& k : kTileDf) consider(k);
-}
-
 // n steps from buffer *cur, which ends as the one that holds the state. With `parity` (ctx_keeps_parity)
 // the launches are even or odd in number as n is.
 cudaError_t advance(const lbm_ctx* c, int n, bool parity, int* cur, int* launches) {
     cudaError_t e = cudaSuccess;
-    if (c->tile_steps > 1 && n > 1) {
-        int parts = (n + c->tile_steps - 1) / c->tile_steps;
-        if (parity && ((parts ^ n) & 1)) ++parts;
-        for (int k = 0; k < parts && e == cudaSuccess; ++k) {
-            const int steps = n / parts + (k < n % parts);
-            e = lbm::launch_tile_steps(c->P, c->scheme, c->tile_region, c->fg[*cur], c->fg[1 - *cur], steps, c->stream);
+    lbm::StepPlan plan{};
+    if (c->P.Q == 9 && n > 1) plan = lbm::plan_steps(c->P.nx, c->P.ny, c->scheme == LBM_SCHEME_FINITE_DIFFERENCE, n, parity, c->sms);
+    if (plan.region) {
+        for (int k = 0; k < plan.parts && e == cudaSuccess; ++k) {
+            const int steps = n / plan.parts + (k < n % plan.parts);
+            e = lbm::launch_tile_steps(c->P, c->scheme, plan.region, c->fg[*cur], c->fg[1 - *cur], steps, c->stream);
             *cur = 1 - *cur;
             *launches += 1;
         }
@@ -367,8 +321,9 @@ int lbm::create_ctx(lbm_ctx** out, const int grid[3], int lattice, double tau_f,
     P.drho_d = rho_ratio - 1.0;
     P.rho2_d = 1.0;
 
-    int rc = LBM_OK, sms = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) == cudaSuccess) plan_steps(c, sms);
+    int rc = LBM_OK;
+    // without the number no plan of several steps per launch fits
+    if (cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) c->sms = 0;
     auto fail = [&](int code) {
         std::snprintf(g_create_error, sizeof g_create_error, "%s", c->err);
         free_ctx(c);

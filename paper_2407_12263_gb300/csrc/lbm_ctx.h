@@ -31,7 +31,7 @@ struct lbm_ctx {
     int graph_launches;               // kernel launches of such a graph
     bool graph_flips;                 // it ends in the other buffer
     bool captured;                    // a caller's capture has recorded a call that holds a buffer's address
-    int tile_region, tile_steps;      // D2Q9: steps per launch at most and their blocks' regions; 1: single steps
+    int sms;                          // SMs of the device, for plan_steps (step_plan.h)
     bool batch_owned;      // a case of an lbm_batch: lbm_destroy leaves it to lbm_batch_destroy
     void* jump_ws;         // surrogate jumps: a backup state, then four coarse field arrays
     size_t jump_ws_bytes;  // (allocated by the first jump or lbm_surrogate_reserve, kept until destroy)

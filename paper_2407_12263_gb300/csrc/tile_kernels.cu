@@ -8,7 +8,7 @@
 // same way: every value is what launches of single steps give, bit for bit.
 //
 // What bounds it is the chain of a step's instructions in a block (0.66 us for 16 x 16 cells, 0.9 for 24 x
-// 24) and 1.5 to 4 us to bring a region up and down; lbm_api.cu has the measured rule by which a
+// 24) and 1.5 to 4 us to bring a region up and down; step_plan.h has the measured rule by which a
 // grid takes this path. 64 x 64 FP32: 1.49 -> 0.96 us per step, the finite-difference variant 2.70 -> 1.39.
 //
 // One thread per cell of the region. A step reads the stencil from shared memory, and writes the new

@@ -1,0 +1,75 @@
+"""The launches of a call's steps on a D2Q9 grid (step_plan.h), compiled for the host: never dearer by the rule's
+own figures than single steps, for every number of steps of a call and not only for many, an even number
+where the parity of the steps asks for one, and within the kernel's limits. The expected plans are those of the
+measured times named beside them.
+"""
+import ctypes
+import subprocess
+from pathlib import Path
+
+import pytest
+
+from paper_2407_12263_gb300 import inputs as I
+from paper_2407_12263_gb300 import lbm
+
+CSRC = Path(__file__).resolve().parent.parent / "paper_2407_12263_gb300" / "csrc"
+SMS = 152
+
+
+@pytest.fixture(scope="module")
+def plan(tmp_path_factory):
+    d = tmp_path_factory.mktemp("plan")
+    (d / "plan.cpp").write_text(f'''#include "{CSRC}/step_plan.h"
+extern "C" double plan(int nx, int ny, int fd, int n, int parity, int sms, int* out) {{
+    const lbm::StepPlan p = lbm::plan_steps(nx, ny, fd, n, parity, sms);
+    out[0] = p.region; out[1] = p.parts;
+    return p.cost;
+}}''')
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-Wall", "-Werror", "-o", d / "plan.so", d / "plan.cpp"], check=True)
+    f = ctypes.CDLL(str(d / "plan.so")).plan
+    f.restype = ctypes.c_double
+    out = (ctypes.c_int * 2)()
+
+    def call(nx, ny, fd, n, parity, sms=SMS):
+        cost = f(nx, ny, fd, n, parity, sms, out)
+        return out[0], out[1], cost
+    return call
+
+
+@pytest.mark.parametrize("fd", [0, 1])
+@pytest.mark.parametrize("grid", [(3, 3), (40, 40), (64, 64), (97, 96), (128, 128), (184, 184), (200, 168), (216, 216), (256, 256), (304, 304),
+                                  (16, 700), (700, 16), (3, 4000), (300, 40), (1200, 1200), (3, 700000000)])
+def test_a_plan_is_never_dearer_than_single_steps(plan, grid, fd):
+    for parity in (0, 1):
+        for n in range(1, 70):
+            region, parts, cost = plan(*grid, fd, n, parity)
+            single = plan(*grid, fd, 1, 0)[2]
+            assert cost <= n * single * (1 + 1e-12)
+            if region:
+                most = -(-n // parts)
+                tile = region - 2 * most * (2 if fd else 1)
+                assert tile >= 4 and parts >= 1 and most >= 1
+                assert not parity or (parts - n) % 2 == 0
+            assert plan(*grid, fd, n, parity, 0)[0] == 0
+
+
+@pytest.mark.parametrize("side,n,parity", [
+    (64, 2, 1),     # two single steps of a captured call 3.1 us, two regions of a step each 4.4
+    (128, 2, 1),    # 3.4 and 6.6
+    (184, 2, 0),    # 4.0 and 4.96
+    (200, 2, 0),    # 4.1 and 5.0
+    (200, 4, 0),    # 8.2 and 9.9
+    (184, 2, 1), (200, 4, 1)])
+def test_short_calls_that_take_single_steps(plan, side, n, parity):
+    assert plan(side, side, 0, n, parity)[0] == 0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("side,n", [(184, 2), (200, 2), (200, 4)])
+def test_short_calls_launch_single_steps(side, n):
+    grid = (side, side, 1)
+    with lbm.Lattice(grid, 9) as g:
+        g.init_phi(I.droplet_phi(grid, side / 4, 4.0))
+        before = g.launch_count
+        g.step(n)
+        assert g.launch_count - before == n
