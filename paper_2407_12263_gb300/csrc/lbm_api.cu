@@ -107,10 +107,10 @@ cudaError_t advance(const lbm_ctx* c, int n, bool parity, int* cur, int* launche
     cudaError_t e = cudaSuccess;
     lbm::StepPlan plan{};
     if (c->P.Q == 9 && n > 1) plan = lbm::plan_steps(c->P.nx, c->P.ny, c->scheme == LBM_SCHEME_FINITE_DIFFERENCE, n, parity, c->sms);
-    if (plan.region) {
+    if (plan.parts) {
         for (int k = 0; k < plan.parts && e == cudaSuccess; ++k) {
             const int steps = n / plan.parts + (k < n % plan.parts);
-            e = lbm::launch_tile_steps(c->P, c->scheme, plan.region, c->fg[*cur], c->fg[1 - *cur], steps, c->stream);
+            e = lbm::launch_tile_steps(c->P, c->scheme, c->fg[*cur], c->fg[1 - *cur], steps, c->stream);
             *cur = 1 - *cur;
             *launches += 1;
         }

@@ -52,11 +52,10 @@ enum StorageKind { STORE_F32 = 0, STORE_F16 = 1, STORE_BF16 = 2 };
 // population and its opposite, so one load serves all four values.
 cudaError_t launch_step(const Params& P, int scheme, const void* fg_in, void* fg_out, float* phi_fd,
                         cudaStream_t s, int* launches);
-// `steps` time steps of a D2Q9 grid in one launch: blocks of region x region threads (16 or 24; 32 for
-// the finite-difference variant) advance tiles of region - 2 reach steps cells,
-// reach = 1 (difference-free) or 2. The same bits as `steps` launches of single steps.
-cudaError_t launch_tile_steps(const Params& P, int scheme, int region, const void* fg_in, void* fg_out, int steps,
-                              cudaStream_t s);
+// `steps` time steps of a D2Q9 grid in one launch: blocks of 16 x 16 threads advance tiles of
+// 16 - 2 reach steps cells, reach = 1 (difference-free) or 2. The same bits as `steps` launches of
+// single steps.
+cudaError_t launch_tile_steps(const Params& P, int scheme, const void* fg_in, void* fg_out, int steps, cudaStream_t s);
 cudaError_t launch_fd_phi(const Params& P, const void* fg_in, float* phi_fd, cudaStream_t s);
 
 // Initial populations for z in [z0, z0 + nzs). phi0s holds planes z0-1 .. z0+nzs of phi0

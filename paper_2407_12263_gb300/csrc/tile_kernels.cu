@@ -1,29 +1,30 @@
 // tile_kernels.cu -- several time steps of a small D2Q9 grid per launch.
 //
 // A step of a small grid is over before the next launch can start: a 64 x 64 step takes 1.5 us, of
-// which the cells' work is less than half. Here a block loads the state of a region of R x R cells into shared
-// memory and advances it `steps` times by itself, the cells it may still use shrinking by the reach of
+// which the cells' work is less than half. Here a block loads the state of a region of 16 x 16 cells into
+// shared memory and advances it `steps` times by itself, the cells it may still use shrinking by the reach of
 // a step (one cell, two in the finite-difference variant: phi, then its gradient) on every side,
 // and stores the tile that is left. Cells of the halo are computed by several blocks, each in the
 // same way: every value is what launches of single steps give, bit for bit.
 //
-// What bounds it is the chain of a step's instructions in a block (0.66 us for 16 x 16 cells, 0.9 for 24 x
-// 24) and 1.5 to 4 us to bring a region up and down; step_plan.h has the measured rule by which a
-// grid takes this path. 64 x 64 FP32: 1.49 -> 0.96 us per step, the finite-difference variant 2.70 -> 1.39.
+// What bounds it is the chain of a step's instructions in a block (0.66 us) and 1.5 us to bring a region up
+// and down; step_plan.h has the measured rule by which a grid takes this path. 64 x 64 FP32: 1.55 -> 1.01 us per
+// step, the finite-difference variant 2.72 -> 1.41, where one launch takes the place of a step's two.
 //
 // One thread per cell of the region. A step reads the stencil from shared memory, and writes the new
 // state back between two barriers, so one copy of the state serves. The arithmetic is that of
 // step_cell (cell.cuh); tile_pull is its propagation with the words taken from shared memory.
 #include "cell.cuh"
+#include "step_plan.h"
 
 namespace lbm {
 
 namespace {
 
-constexpr int Q9 = 9;
+constexpr int Q9 = 9, R = kTileSide;
 
-// pull (cell.cuh) in storage units, from the words and moments of a region of `n` cells in shared memory;
-// o: offsets of the eight neighbours' cells.
+// pull (cell.cuh) in storage units, from the words and moments of a region of `n` cells in shared memory,
+// whose rows lie as nb says.
 template <int S, bool WALLS>
 __device__ __forceinline__ void tile_pull(const Params& P, const typename Store<S>::Word* words, const float2* moments, int n, int c,
                                           const Nbr& nb, float (&fb)[Q9], float (&gb)[Q9], int& phi_fx, const WallSide& ws) {
@@ -74,13 +75,13 @@ __device__ __forceinline__ void tile_gradient(const float* phi, int c, const Nbr
     gz *= 3.f;
 }
 
-template <int R, int S, int SCHEME>
+template <int S, int SCHEME>
 constexpr size_t tile_smem() {
     return (size_t)R * R * (sizeof(float2) + Lat<Q9>::kPairs * sizeof(typename Store<S>::Word) + (SCHEME == SCHEME_FD ? sizeof(float) : 0));
 }
 
-template <int R, int SCHEME, bool GEN, int S>
-__global__ void __launch_bounds__(R* R)
+template <int SCHEME, bool GEN, int S>
+__global__ void __launch_bounds__(R* R, kTileResident)
 tile_step_kernel(const Params P, const void* fg_in, void* __restrict__ fg_out, int steps) {
     using Word = typename Store<S>::Word;
     constexpr int n = R * R, kReach = SCHEME == SCHEME_FD ? 2 : 1;
@@ -155,20 +156,19 @@ tile_step_kernel(const Params P, const void* fg_in, void* __restrict__ fg_out, i
     }
 }
 
-template <int R, int SCHEME, bool GEN, int S>
+template <int SCHEME, bool GEN, int S>
 cudaError_t launch_tile(const Params& P, const void* in, void* out, int steps, cudaStream_t s) {
-    constexpr size_t smem = tile_smem<R, S, SCHEME>();
+    constexpr size_t smem = tile_smem<S, SCHEME>();
     const int tile = R - 2 * steps * (SCHEME == SCHEME_FD ? 2 : 1);
     if (steps < 1 || tile < 1) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(tile_step_kernel<R, SCHEME, GEN, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    static_assert(smem <= 48 << 10, "larger needs cudaFuncSetAttribute");
     const dim3 grid((P.nx + tile - 1) / tile, (P.ny + tile - 1) / tile);
-    return launch_chained(tile_step_kernel<R, SCHEME, GEN, S>, grid, dim3(R * R), smem, s, P, in, out, steps);
+    return launch_chained(tile_step_kernel<SCHEME, GEN, S>, grid, dim3(R * R), smem, s, P, in, out, steps);
 }
 
-template <int R, int SCHEME>
-cudaError_t launch_tile_r(const Params& P, const void* in, void* out, int steps, cudaStream_t s) {
-#define LBM_TILE(S) (P.general ? launch_tile<R, SCHEME, true, S>(P, in, out, steps, s) : launch_tile<R, SCHEME, false, S>(P, in, out, steps, s))
+template <int SCHEME>
+cudaError_t launch_tile_s(const Params& P, const void* in, void* out, int steps, cudaStream_t s) {
+#define LBM_TILE(S) (P.general ? launch_tile<SCHEME, true, S>(P, in, out, steps, s) : launch_tile<SCHEME, false, S>(P, in, out, steps, s))
     if (P.storage == STORE_F16) return LBM_TILE(STORE_F16);
     if (P.storage == STORE_BF16) return LBM_TILE(STORE_BF16);
     return LBM_TILE(STORE_F32);
@@ -177,17 +177,9 @@ cudaError_t launch_tile_r(const Params& P, const void* in, void* out, int steps,
 
 }  // namespace
 
-cudaError_t launch_tile_steps(const Params& P, int scheme, int region, const void* in, void* out, int steps, cudaStream_t s) {
+cudaError_t launch_tile_steps(const Params& P, int scheme, const void* in, void* out, int steps, cudaStream_t s) {
     if (P.Q != 9) return cudaErrorInvalidValue;
-    if (scheme == SCHEME_DF) {
-        if (region == 16) return launch_tile_r<16, SCHEME_DF>(P, in, out, steps, s);
-        if (region == 24) return launch_tile_r<24, SCHEME_DF>(P, in, out, steps, s);
-    } else {
-        if (region == 16) return launch_tile_r<16, SCHEME_FD>(P, in, out, steps, s);
-        if (region == 24) return launch_tile_r<24, SCHEME_FD>(P, in, out, steps, s);
-        if (region == 32) return launch_tile_r<32, SCHEME_FD>(P, in, out, steps, s);
-    }
-    return cudaErrorInvalidValue;
+    return scheme == SCHEME_DF ? launch_tile_s<SCHEME_DF>(P, in, out, steps, s) : launch_tile_s<SCHEME_FD>(P, in, out, steps, s);
 }
 
 }  // namespace lbm

@@ -22,17 +22,17 @@ def plan(tmp_path_factory):
     (d / "plan.cpp").write_text(f'''#include "{CSRC}/step_plan.h"
 extern "C" double plan(int nx, int ny, int fd, int n, int parity, int sms, int* out) {{
     const lbm::StepPlan p = lbm::plan_steps(nx, ny, fd, n, parity, sms);
-    out[0] = p.region; out[1] = p.parts;
+    *out = p.parts;
     return p.cost;
 }}''')
     subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-Wall", "-Werror", "-o", d / "plan.so", d / "plan.cpp"], check=True)
     f = ctypes.CDLL(str(d / "plan.so")).plan
     f.restype = ctypes.c_double
-    out = (ctypes.c_int * 2)()
+    out = ctypes.c_int()
 
     def call(nx, ny, fd, n, parity, sms=SMS):
-        cost = f(nx, ny, fd, n, parity, sms, out)
-        return out[0], out[1], cost
+        cost = f(nx, ny, fd, n, parity, sms, ctypes.byref(out))
+        return out.value, cost
     return call
 
 
@@ -42,12 +42,12 @@ extern "C" double plan(int nx, int ny, int fd, int n, int parity, int sms, int* 
 def test_a_plan_is_never_dearer_than_single_steps(plan, grid, fd):
     for parity in (0, 1):
         for n in range(1, 70):
-            region, parts, cost = plan(*grid, fd, n, parity)
-            single = plan(*grid, fd, 1, 0)[2]
+            parts, cost = plan(*grid, fd, n, parity)
+            single = plan(*grid, fd, 1, 0)[1]
             assert cost <= n * single * (1 + 1e-12)
-            if region:
+            if parts:
                 most = -(-n // parts)
-                tile = region - 2 * most * (2 if fd else 1)
+                tile = 16 - 2 * most * (2 if fd else 1)
                 assert tile >= 4 and parts >= 1 and most >= 1
                 assert not parity or (parts - n) % 2 == 0
             assert plan(*grid, fd, n, parity, 0)[0] == 0
@@ -62,6 +62,13 @@ def test_a_plan_is_never_dearer_than_single_steps(plan, grid, fd):
     (184, 2, 1), (200, 4, 1)])
 def test_short_calls_that_take_single_steps(plan, side, n, parity):
     assert plan(side, side, 0, n, parity)[0] == 0
+
+
+# launches for 32 steps; 0 where four handles side by side are faster with single steps
+@pytest.mark.parametrize("side,fd,parts", [(64, 0, 7), (96, 0, 8), (128, 0, 16), (184, 0, 0), (216, 0, 0),
+                                           (64, 1, 16), (96, 1, 16), (128, 1, 16), (184, 1, 32), (216, 1, 0)])
+def test_plans_leave_room_for_other_handles(plan, side, fd, parts):
+    assert plan(side, side, fd, 32, 0)[0] == parts
 
 
 @pytest.mark.gpu
