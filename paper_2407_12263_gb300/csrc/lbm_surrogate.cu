@@ -531,7 +531,7 @@ int lbm_surrogate_jump(lbm_ctx* c, lbm_net* n, int f, const float mean_std[10], 
     if (proj) {
         if ((rc = cu(lbm::launch_project_solenoidal(pred + nc, grid_c[0], grid_c[1], grid_c[2], proj, c->stream))))
             return rc;
-        c->launches += 9;
+        c->launches += lbm::kProjectLaunches;
         rep->projected = 1;
     }
     // 2. mass and interface position of the prediction, measured on the coarse grid

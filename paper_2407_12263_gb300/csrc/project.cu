@@ -170,7 +170,7 @@ cudaError_t dft(float2* W, const float2* tw, const float* in_real, float* out_re
 
 }  // namespace proj
 
-// The whole projection of u [3][nz][ny][nx] in place: 8 launches on stream s.
+// The whole projection of u [3][nz][ny][nx] in place: kProjectLaunches launches on stream s.
 cudaError_t launch_project_solenoidal(float* u, int nx, int ny, int nz, void* work, cudaStream_t s) {
     using namespace proj;
     float2* tw = static_cast<float2*>(work);

@@ -106,6 +106,7 @@ cudaError_t launch_l1_difference(const float* a, const float* b, long long n, do
 //   out[3]  = max(out[3], largest |u|^2 of start and prediction) (as non-negative double bits).
 cudaError_t launch_jump_measures(const float* start, const float* pred, int ncx, int ncy, int ncz, int walls, double* out,
                                  cudaStream_t s);
+constexpr int kProjectLaunches = 8;  // twiddles, three passes, the modes, three passes back
 // The divergence-free part of the periodic velocity u [3][nz][ny][nx] in place
 // (lbm_project_solenoidal); work holds project_workspace_bytes() bytes, 16-byte aligned.
 cudaError_t launch_project_solenoidal(float* u, int nx, int ny, int nz, void* work, cudaStream_t s);
