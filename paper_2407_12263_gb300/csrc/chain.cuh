@@ -41,7 +41,9 @@ cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, siz
     cfg.stream = s;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+    if (e != cudaSuccess) (void)cudaGetLastError();  // reported here: the next plain launch must not find it
+    return e;
 }
 
 }  // namespace lbm

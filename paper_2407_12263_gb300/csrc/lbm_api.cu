@@ -102,23 +102,28 @@ void drop_graphs(lbm_ctx* c) {
 }
 
 // n steps from buffer *cur, which ends as the one that holds the state. With `parity` (ctx_keeps_parity)
-// the launches are even or odd in number as n is.
+// the launches are even or odd in number as n is. After an error *cur and *launches are those of the steps
+// that were launched.
 cudaError_t advance(const lbm_ctx* c, int n, bool parity, int* cur, int* launches) {
     cudaError_t e = cudaSuccess;
     lbm::StepPlan plan{};
     if (c->P.Q == 9 && n > 1) plan = lbm::plan_steps(c->P.nx, c->P.ny, c->scheme == LBM_SCHEME_FINITE_DIFFERENCE, n, parity, c->sms);
     if (plan.parts) {
-        for (int k = 0; k < plan.parts && e == cudaSuccess; ++k) {
+        for (int k = 0; k < plan.parts; ++k) {
             const int steps = n / plan.parts + (k < n % plan.parts);
             e = lbm::launch_tile_steps(c->P, c->scheme, c->fg[*cur], c->fg[1 - *cur], steps, c->stream);
+            if (e != cudaSuccess) return e;
             *cur = 1 - *cur;
             *launches += 1;
         }
         return e;
     }
-    for (int k = 0; k < n && e == cudaSuccess; ++k) {
-        e = lbm::launch_step(c->P, c->scheme, c->fg[*cur], c->fg[1 - *cur], c->phi_fd, c->stream, launches);
+    for (int k = 0; k < n; ++k) {
+        int of_step = 0;
+        e = lbm::launch_step(c->P, c->scheme, c->fg[*cur], c->fg[1 - *cur], c->phi_fd, c->stream, &of_step);
+        if (e != cudaSuccess) return e;
         *cur = 1 - *cur;
+        *launches += of_step;
     }
     return e;
 }
@@ -140,6 +145,7 @@ int capture_graph(lbm_ctx* c, int start) {
     if (graph) cudaGraphDestroy(graph);
     if (e != cudaSuccess) {
         c->graph_exec[start] = nullptr;
+        (void)cudaGetLastError();  // ending the capture leaves it too: the next plain launch must not find it
         return set_error(c, LBM_ECUDA, "capturing the step graph failed: %s", cudaGetErrorString(e));
     }
     return LBM_OK;

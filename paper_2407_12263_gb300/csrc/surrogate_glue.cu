@@ -416,24 +416,23 @@ cudaError_t launch_balance(const Params& P, void* fg, const RestartSums& sums, c
 }
 
 template <int F>
-static void coarse_phi_f(const Params& P, void* fg, const RestartSums* sums, float* out, cudaStream_t s) {
+static cudaError_t coarse_phi_f(const Params& P, void* fg, const RestartSums* sums, float* out, cudaStream_t s) {
     const dim3 block(32, 4), grid((P.nx + 31) / 32, (P.ny / F + 3) / 4, P.nz / F);
     const Balance B = balance_of_restart(P, sums);
-    (void)launch_chained(sums ? coarse_phi_kernel<F, true> : coarse_phi_kernel<F, false>, grid, block, 0, s, moment_plane(fg), P.nx,
+    return launch_chained(sums ? coarse_phi_kernel<F, true> : coarse_phi_kernel<F, false>, grid, block, 0, s, moment_plane(fg), P.nx,
                          P.ny, P.nz, B, out);
 }
 
 cudaError_t launch_coarse_phi(const Params& P, void* fg, int factor, const RestartSums* sums, float* out, cudaStream_t s) {
     switch (factor) {
-        case 1: coarse_phi_f<1>(P, fg, sums, out, s); break;
-        case 2: coarse_phi_f<2>(P, fg, sums, out, s); break;
-        case 4: coarse_phi_f<4>(P, fg, sums, out, s); break;
-        case 8: coarse_phi_f<8>(P, fg, sums, out, s); break;
-        case 16: coarse_phi_f<16>(P, fg, sums, out, s); break;
-        case 32: coarse_phi_f<32>(P, fg, sums, out, s); break;
+        case 1: return coarse_phi_f<1>(P, fg, sums, out, s);
+        case 2: return coarse_phi_f<2>(P, fg, sums, out, s);
+        case 4: return coarse_phi_f<4>(P, fg, sums, out, s);
+        case 8: return coarse_phi_f<8>(P, fg, sums, out, s);
+        case 16: return coarse_phi_f<16>(P, fg, sums, out, s);
+        case 32: return coarse_phi_f<32>(P, fg, sums, out, s);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 // Where fine coordinate i (of n = nc f cells) falls between coarse cell centres: the two coarse
