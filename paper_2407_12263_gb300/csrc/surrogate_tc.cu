@@ -261,14 +261,15 @@ struct ConvArgs {
 
 // The running sum of w diff^2 of a thread, as an unevaluated pair of FP32 (exact products by FMA,
 // two-sums: about 48 bits; an FP64 multiply-add per element would take as long as the layer's
-// MMAs). Values whose square may leave the FP32 range go to an FP64 sum.
+// MMAs). An FP64 sum takes the values whose products, their rounding errors (2^-24 of them) or sums over 2^31
+// elements may leave the FP32 range.
 struct LossSum {
     float hi = 0.f, lo = 0.f;
     double far = 0.0;
     __device__ __forceinline__ void add(float w, float d) {
         const float m = fabsf(d);
         if (m == 0.f) return;
-        if (!(m > 1e-12f && m < 1e12f && w < 1e12f && (w > 1e-12f || w == 0.f))) {
+        if (!(m > 1e-9f && m < 1e9f && w < 1e9f && (w > 1e-9f || w == 0.f))) {
             far += (double)w * (double)d * (double)d;
             return;
         }
