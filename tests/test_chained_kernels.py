@@ -19,7 +19,7 @@ def functions(csrc):
     for path in sorted(csrc.glob("*.cu*")):
         text = re.sub(r"//[^\n]*|/\*.*?\*/", "", path.read_text(), flags=re.S)
         for m in re.finditer(r"\b(\w+)\s*\(((?:[^(){};]|\{\}|\([^(){};]*\))*)\)\s*(?:const\s*)?\{", text):
-            if m.group(1) in ("if", "for", "while", "switch", "__launch_bounds__"):
+            if m.group(1) in ("if", "for", "while", "switch", "constexpr", "__launch_bounds__"):
                 continue
             depth, i = 1, m.end()
             while depth and i < len(text):
