@@ -17,28 +17,21 @@
 // and writes the phi plane; the second is the fused step with grad phi taken from the
 // isotropic central difference of that plane instead of K1.
 #include "cell.cuh"
+#include "step_plan.h"
 
 namespace lbm {
 
-// Thread block: 128 threads, one cell per thread, x fastest (step_shape has the shapes). With FP32 storage the register budget allows 4
+// Thread block: 128 threads, one cell per thread, x fastest (step_shape in step_plan.h has the shapes). With FP32 storage the register budget allows 4
 // blocks (16 warps) per SM: the difference-free step needs ~122 registers and runs at that
 // occupancy with every (f, g) load of a cell in flight. A 16-bit cell moves half the bytes, so
 // the same bandwidth needs more cells in flight: the 16-bit steps are held to 96 registers for
 // 5 blocks (20 warps), which they fit without spilling.
-constexpr int kStepThreads = 128;
 constexpr int LBM_STEP_MINB = 4;
 
 template <int S>
 constexpr int step_min_blocks() {
     return S == STORE_F32 ? LBM_STEP_MINB : 5;
 }
-
-// i / nx (nx > 1) for i < 2^31 as a product: mul = ceil(2^(32 + shift) / nx), 2^shift < nx <= 2^(shift + 1). The
-// excess mul nx - 2^(32 + shift) is below nx <= 2^(shift + 1), so i times it stays below 2^(32 + shift).
-struct RowDiv {
-    unsigned mul;
-    int shift;
-};
 
 // The cell of a thread, false beyond the grid. PACK: blocks of 128 cells that follow one another in
 // a plane, whatever its rows, instead of blocks of whole rows or of 32 x 4 cells.
@@ -56,9 +49,6 @@ __device__ __forceinline__ bool own_cell(const Params& P, const RowDiv& d, int& 
     return x < P.nx && y < P.ny;
 }
 
-// How a step's blocks lie and address: whole rows or 32 x 4 cells, packed, or whole blocks with 64-bit
-// addresses for the 16-bit D3Q19 planes of 4 GiB and more (2^29 cells), where a byte offset does not fit.
-enum StepForm { WHOLE = 0, PACKED = 1, WIDE = 2 };
 template <int Q, int S>
 constexpr bool narrow_form(int form) { return Q == 19 && S != STORE_F32 && form != WIDE; }
 
@@ -87,42 +77,15 @@ fd_phi_kernel(const Params P, const void* fg_in, float* __restrict__ phi, const 
     phi[c] = gb[0];
 }
 
-// Blocks of one 128-cell row where rows are at least that long, else 32 x 4 (a warp spans 32 consecutive
-// cells of a row either way); where such blocks would stand over the grid's edges, packed ones, which
-// leave no lane idle but in a plane's last block. Packed blocks cost a product per cell to find the
-// row: 0.4% at 128^3 (59.98 against 60.36 us FP16, 93.16 against 93.39 FP32), so whole blocks stay where
-// they fit. Where they do not, packed ones were faster at every size tried (us per step):
-//   grid              33^3  33^3   97x96x96  126^3  130^3  130^3   200^3   200^3   94x75x301  600^2  330x270
-//                     FP16  FP32*  FP32*     FP16   FP16   FP32    BF16    FP32    BF16*      FP32   FP32
-//   whole blocks      3.31  4.30   51.2      61.1   84.6   115.5   266.0   373.6   74.1       6.13   2.87
-//   packed            2.42  3.30   44.0      60.0   65.7   99.7    231.2   349.1   72.6       5.85   2.65
-// (* walls and a density ratio)
-struct StepShape {
-    dim3 block, grid;
-    StepForm form;
-    RowDiv d;
-};
-
 static StepShape step_shape(const Params& P) {
-    StepShape h;
-    h.block = P.nx >= 128 ? dim3(128, 1, 1) : dim3(32, 4, 1);
-    h.grid = dim3((P.nx + h.block.x - 1) / h.block.x, (P.ny + h.block.y - 1) / h.block.y, P.nz);
-    const unsigned blocks = ((unsigned)P.nxy + kStepThreads - 1) / kStepThreads;
-    h.form = P.nx > 1 && blocks < h.grid.x * h.grid.y ? PACKED : WHOLE;
-    if (P.Q == 19 && P.storage != STORE_F32 && P.N >= (1ll << 29)) h.form = WIDE;
-    h.d = RowDiv{0u, 0};
-    if (h.form == PACKED) {
-        h.block = dim3(kStepThreads, 1, 1);
-        h.grid = dim3(blocks, 1, P.nz);
-        while ((2 << h.d.shift) < P.nx) ++h.d.shift;
-        h.d.mul = (unsigned)(((1ull << (32 + h.d.shift)) + P.nx - 1) / P.nx);
-    }
-    return h;
+    return step_shape(P.nx, P.ny, P.nz, P.Q == 19 && P.storage != STORE_F32);
 }
+static dim3 grid_of(const StepShape& h) { return dim3(h.grid[0], h.grid[1], h.grid[2]); }
+static dim3 block_of(const StepShape& h) { return dim3(h.block[0], h.block[1]); }
 
 template <int Q, int S, int FORM>
 static cudaError_t fd_phi_qs(const Params& P, const StepShape& h, const void* in, float* phi, cudaStream_t s) {
-    return launch_chained(P.walls ? fd_phi_kernel<Q, S, true, FORM> : fd_phi_kernel<Q, S, false, FORM>, h.grid, h.block, 0, s, P, in,
+    return launch_chained(P.walls ? fd_phi_kernel<Q, S, true, FORM> : fd_phi_kernel<Q, S, false, FORM>, grid_of(h), block_of(h), 0, s, P, in,
                           phi, h.d);
 }
 
@@ -132,13 +95,13 @@ static cudaError_t step_qs(const Params& P, const StepShape& h, int scheme, cons
     if (scheme == SCHEME_DF) {
         *launches += 1;
         return launch_chained(P.general ? step_kernel<Q, SCHEME_DF, true, S, FORM> : step_kernel<Q, SCHEME_DF, false, S, FORM>,
-                              h.grid, h.block, 0, s, P, in, out, (const float*)nullptr, h.d);
+                              grid_of(h), block_of(h), 0, s, P, in, out, (const float*)nullptr, h.d);
     }
     *launches += 2;
     const cudaError_t e = fd_phi_qs<Q, S, FORM>(P, h, in, phi, s);
     if (e != cudaSuccess) return e;
-    return launch_chained(P.general ? step_kernel<Q, SCHEME_FD, true, S, FORM> : step_kernel<Q, SCHEME_FD, false, S, FORM>, h.grid,
-                          h.block, 0, s, P, in, out, (const float*)phi, h.d);
+    return launch_chained(P.general ? step_kernel<Q, SCHEME_FD, true, S, FORM> : step_kernel<Q, SCHEME_FD, false, S, FORM>, grid_of(h),
+                          block_of(h), 0, s, P, in, out, (const float*)phi, h.d);
 }
 
 template <int Q, int S>

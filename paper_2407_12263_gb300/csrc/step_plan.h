@@ -1,11 +1,59 @@
-// step_plan.h -- how the steps of a call are launched on a D2Q9 grid: one by one, or several per launch
-// (tile_kernels.cu). Host code without CUDA.
+// step_plan.h -- how steps are launched: the blocks of a single step (step_kernels.cu), and on a D2Q9 grid how many
+// steps of a call share a launch (tile_kernels.cu). Host code without CUDA.
 #pragma once
 
 #include <algorithm>
 #include <cmath>
 
 namespace lbm {
+
+constexpr int kStepThreads = 128;  // of a block of a single step, one cell each
+
+// i / nx (nx > 1) for i < 2^31 as a product, the high word of i mul shifted right by `shift`: mul =
+// ceil(2^(32 + shift) / nx), 2^shift < nx <= 2^(shift + 1). The excess mul nx - 2^(32 + shift) is below nx <=
+// 2^(shift + 1), so i times it stays below 2^(32 + shift).
+struct RowDiv {
+    unsigned mul;
+    int shift;
+};
+
+// How a step's blocks lie and address: whole rows or 32 x 4 cells, packed, or whole blocks with 64-bit
+// addresses for the 16-bit D3Q19 planes of 4 GiB and more (2^29 cells), where a byte offset does not fit.
+enum StepForm { WHOLE = 0, PACKED = 1, WIDE = 2 };
+
+// Blocks of one 128-cell row where rows are at least that long, else 32 x 4 (a warp spans 32 consecutive
+// cells of a row either way); where such blocks would stand over the grid's edges, packed ones, which
+// leave no lane idle but in a plane's last block. Packed blocks cost a product per cell to find the
+// row: 0.4% at 128^3 (59.98 against 60.36 us FP16, 93.16 against 93.39 FP32), so whole blocks stay where
+// they fit. Where they do not, packed ones were faster at every size tried (us per step):
+//   grid              33^3  33^3   97x96x96  126^3  130^3  130^3   200^3   200^3   94x75x301  600^2  330x270
+//                     FP16  FP32*  FP32*     FP16   FP16   FP32    BF16    FP32    BF16*      FP32   FP32
+//   whole blocks      3.31  4.30   51.2      61.1   84.6   115.5   266.0   373.6   74.1       6.13   2.87
+//   packed            2.42  3.30   44.0      60.0   65.7   99.7    231.2   349.1   72.6       5.85   2.65
+// (* walls and a density ratio)
+struct StepShape {
+    unsigned block[2], grid[3];
+    StepForm form;
+    RowDiv d;
+};
+
+inline StepShape step_shape(int nx, int ny, int nz, bool d3q19_16bit) {
+    StepShape h{{nx >= 128 ? 128u : 32u, nx >= 128 ? 1u : 4u}, {0u, 0u, (unsigned)nz}, WHOLE, {0u, 0}};
+    h.grid[0] = (nx + h.block[0] - 1) / h.block[0];
+    h.grid[1] = (ny + h.block[1] - 1) / h.block[1];
+    const unsigned blocks = ((unsigned)nx * (unsigned)ny + kStepThreads - 1) / kStepThreads;
+    if (nx > 1 && blocks < h.grid[0] * h.grid[1]) h.form = PACKED;
+    if (d3q19_16bit && (long long)nx * ny * nz >= (1ll << 29)) h.form = WIDE;
+    if (h.form == PACKED) {
+        h.block[0] = kStepThreads;
+        h.block[1] = 1;
+        h.grid[0] = blocks;
+        h.grid[1] = 1;
+        while ((2ll << h.d.shift) < nx) ++h.d.shift;
+        h.d.mul = (unsigned)(((1ull << (32 + h.d.shift)) + nx - 1) / nx);
+    }
+    return h;
+}
 
 constexpr int kTileSide = 16;  // cells squared of a block's region
 constexpr int kTileResident = 3;  // such blocks on an SM at once (256 threads of up to 80 registers)

@@ -1,7 +1,8 @@
-"""The launches of a call's steps on a D2Q9 grid (step_plan.h), compiled for the host: never dearer by the rule's
+"""step_plan.h compiled for the host. The launches of a call's steps on a D2Q9 grid: never dearer by the rule's
 own figures than single steps, for every number of steps of a call and not only for many, an even number
-where the parity of the steps asks for one, and within the kernel's limits. The expected plans are those of the
-measured times named beside them.
+where the parity of the steps asks for one, and within the kernel's limits; the expected plans are those of the
+measured times named beside them. The blocks of a single step: every cell of a plane in one lane, and 64-bit
+addresses from 2^29 cells on.
 """
 import ctypes
 import subprocess
@@ -17,16 +18,26 @@ SMS = 152
 
 
 @pytest.fixture(scope="module")
-def plan(tmp_path_factory):
+def library(tmp_path_factory):
     d = tmp_path_factory.mktemp("plan")
     (d / "plan.cpp").write_text(f'''#include "{CSRC}/step_plan.h"
 extern "C" double plan(int nx, int ny, int fd, int n, int parity, int sms, int* out) {{
     const lbm::StepPlan p = lbm::plan_steps(nx, ny, fd, n, parity, sms);
     *out = p.parts;
     return p.cost;
+}}
+extern "C" void shape(int nx, int ny, int nz, int narrow, unsigned* out) {{
+    const lbm::StepShape h = lbm::step_shape(nx, ny, nz, narrow);
+    const unsigned v[] = {{h.block[0], h.block[1], h.grid[0], h.grid[1], h.grid[2], (unsigned)h.form, h.d.mul, (unsigned)h.d.shift}};
+    for (int k = 0; k < 8; ++k) out[k] = v[k];
 }}''')
     subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-Wall", "-Werror", "-o", d / "plan.so", d / "plan.cpp"], check=True)
-    f = ctypes.CDLL(str(d / "plan.so")).plan
+    return ctypes.CDLL(str(d / "plan.so"))
+
+
+@pytest.fixture(scope="module")
+def plan(library):
+    f = library.plan
     f.restype = ctypes.c_double
     out = ctypes.c_int()
 
@@ -34,6 +45,42 @@ extern "C" double plan(int nx, int ny, int fd, int n, int parity, int sms, int* 
         cost = f(nx, ny, fd, n, parity, sms, ctypes.byref(out))
         return out.value, cost
     return call
+
+
+@pytest.fixture(scope="module")
+def shape(library):
+    def call(nx, ny, nz, narrow):
+        out = (ctypes.c_uint * 8)()
+        library.shape(nx, ny, nz, narrow, out)
+        return dict(zip(("bx", "by", "gx", "gy", "gz", "form", "mul", "shift"), out))
+    return call
+
+
+WHOLE, PACKED, WIDE = 0, 1, 2
+
+
+@pytest.mark.parametrize("ny", [3, 20, 129])
+def test_step_blocks_cover_a_plane(shape, ny):
+    for nx in list(range(3, 3000)) + [65535, 65537, 1 << 20, (1 << 20) + 1, 5000011, 16000001]:
+        h = shape(nx, ny, 5, 0)
+        assert h["bx"] * h["by"] == 128 and h["gz"] == 5
+        if h["form"] == WHOLE:
+            assert h["gx"] * h["bx"] >= nx > (h["gx"] - 1) * h["bx"] and h["gy"] * h["by"] >= ny > (h["gy"] - 1) * h["by"]
+            assert h["gx"] * h["gy"] == -(-nx * ny // 128)
+        else:
+            assert h["form"] == PACKED and h["gy"] == 1 and h["gx"] * 128 >= nx * ny > (h["gx"] - 1) * 128
+            # the row of a cell, at the ends of rows and of the plane and of the largest plane
+            last = (1 << 31) - 1
+            for i in (0, nx - 1, nx, 2 * nx - 1, nx * ny - 1, nx * ny, last // nx * nx - 1, last // nx * nx, last):
+                assert (i * h["mul"] >> 32) >> h["shift"] == i // nx
+
+
+@pytest.mark.parametrize("grid,narrow,form", [((512, 512, 2048), 1, WIDE), ((512, 512, 2047), 1, WHOLE), ((512, 512, 2048), 0, WHOLE),
+                                              ((1000, 700, 766), 1, PACKED), ((1000, 700, 767), 1, WIDE), ((1000, 700, 767), 0, PACKED),
+                                              ((1 << 29, 3, 1), 0, WHOLE), ((700000001, 3, 1), 0, PACKED)])
+def test_step_form_around_2_to_the_29_cells(shape, grid, narrow, form):
+    assert shape(*grid, narrow)["form"] == form
+    assert narrow == 0 or (form == WIDE) == (grid[0] * grid[1] * grid[2] >= 1 << 29)
 
 
 @pytest.mark.parametrize("fd", [0, 1])
