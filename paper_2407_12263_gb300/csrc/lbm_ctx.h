@@ -21,7 +21,7 @@ struct lbm_ctx {
     float* phi_fd;         // propagated phi plane of the finite-difference variant
     double* partials;      // per-block FP64 partial sums of the mass reduction
     int n_partials;
-    double* result;        // 3 doubles: sum phi, sum rho phi, non-finite count
+    double* result;        // 4 doubles: sum phi, sum rho phi, non-finite count, fixed-point sum of phi (integer bits)
     double* staging;       // FP64 staging for host transfers, allocated on first use
     size_t staging_elems;
     bool initialised;
@@ -33,7 +33,7 @@ struct lbm_ctx {
     bool captured;                    // a caller's capture has recorded a call that holds a buffer's address
     int sms;                          // SMs of the device, for plan_steps (step_plan.h)
     bool batch_owned;      // a case of an lbm_batch: lbm_destroy leaves it to lbm_batch_destroy
-    void* jump_ws;         // surrogate jumps: a backup state, then four coarse field arrays
+    void* jump_ws;         // surrogate jumps: a third state buffer, four coarse field arrays, measures, projection scratch
     size_t jump_ws_bytes;  // (allocated by the first jump or lbm_surrogate_reserve, kept until destroy)
     long long version;     // bumped whenever the parameters or the whole state are replaced
     char err[512];
