@@ -10,7 +10,7 @@
  * FP32 storage), then one plane of words [nz][ny][nx] per opposite pair of populations (i, and
  * j with e_j = -e_i): per cell the pair of i then that of j, 16 B for FP32, 8 B for 16-bit.
  * Every step is one fused stream-collide kernel launch (difference-free scheme), or two
- * launches for the finite-difference variant; several steps of a small D2Q9 grid share one.
+ * launches for the finite-difference variant; on small D2Q9 grids both, or several steps, share one.
  *
  * Units are lattice units: dx = 1 and dt = 1 in every collision, moment and forcing
  * formula; the Courant number only enters the Lax-Wendroff propagation (Sec. 2.2).
@@ -162,16 +162,16 @@ int lbm_init_fields(lbm_ctx *ctx, const double *phi0, const double *u0, const do
  * buffers (lbm_create_ext) and on a case of a batch, the state changes its buffer with every step: what may
  * stand between capture and replay, and between two replays, is any calls that make an even number
  * of steps in all (whatever number each of them makes), initialisations and restarts, and surrogate jumps:
- * accepted ones end in the buffer they began in, a rejected one counts as its k steps. A graph of an
- * odd number of steps is replayed an even number of times. */
+ * accepted ones end in the buffer they began in, a rejected one counts as its k steps. The handle does not
+ * see a replay: a graph that is replayed more than once holds an even number of steps. */
 int lbm_step(lbm_ctx *ctx, int n);
 
 /* Capture the step graph that lbm_step replays from the current state's buffer (and the one from the
  * other buffer, where a replay ends there), if it is not captured yet, and upload it to the device,
  * without running it: the state does not change and no launch is counted. A later lbm_step(n) with n a
  * multiple of graph_steps from this buffer then replays it with no capture and no first-launch
- * upload. Synchronous. LBM_EINVAL if the
- * handle replays no graphs (graph_steps 0), LBM_ESTATE before lbm_init_phi. */
+ * upload. Synchronous. LBM_EINVAL if the handle replays no graphs (graph_steps 0), LBM_ESTATE before
+ * lbm_init_phi. */
 int lbm_graph_prepare(lbm_ctx *ctx);
 
 /*
@@ -238,7 +238,8 @@ int lbm_set_pops(lbm_ctx *ctx, const double *f, const double *g);
 
 /* Kernel launches issued by this handle since creation (one per step for the
  * difference-free scheme, two for the finite-difference variant, plus auxiliaries; on small D2Q9
- * grids, where a launch would take longer than its step, one for several steps). */
+ * grids, where a launch would take longer than its step, one for several steps or for both launches
+ * of a finite-difference step). */
 long long lbm_launch_count(const lbm_ctx *ctx);
 
 /* tau_phi the handle resolved from (tau_g, M). */
